@@ -172,8 +172,9 @@ qla_status qla_get_state(qla_ctx *ctx, double *q_host);
 /* Advance n_steps >= 0 steps of Eq. 2e14 on the context's stream (returns
  * without waiting).  n_steps == 0 is a no-op; otherwise QLA_ESTATE before
  * both a medium and a state are set.  The steps run as one launch each, or
- * (FP32 E_z contexts on large lattices, see qla_set_step_kernel) as one
- * dataflow launch for the whole call; the results are the same bits. */
+ * as one launch for the whole call (dataflow steps of FP32 E_z contexts on
+ * large lattices, resident tiles on small ones, see qla_set_step_kernel);
+ * the results are the same bits. */
 qla_status qla_step(qla_ctx *ctx, long long n_steps);
 
 /* Total energy, Eq. A13 without the cell area: the sum over sites and
@@ -262,7 +263,7 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * qla_set_march_tuning: nx a multiple of 4 for the packed-pair layout, of
  * the per-lane column count otherwise; a window of 64 or 32 x lane columns
  * no wider than nx) and ny >= 8, and the
- * shared-memory tile kernel otherwise.  QLA_KERNEL_TILE / QLA_KERNEL_MARCH
+ * tile kernel otherwise and on small lattices.  QLA_KERNEL_TILE / QLA_KERNEL_MARCH
  * force one (QLA_EINVAL if the marching kernel does not support the
  * lattice, including one whose live planes exceed its 32-bit element
  * offsets: planes x ny x padded nx > 2^32).  Both compute the same operator sequence; FP64 results agree to
@@ -277,6 +278,13 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * marching step after qla_set_medium or a tuning change classifies the
  * items (one small kernel and one synchronisation of the context's
  * stream), so it must not be the first call inside a stream capture.
+ * Small lattices (QLA_KERNEL_AUTO; FP32 up to about 700^2 sites, FP64 as far
+ * as one tile per SM goes, double-single contexts excepted): a qla_step call
+ * runs all its steps in one cooperative launch of the tile kernel, every
+ * tile waiting for its eight neighbours between steps; the results are those
+ * of one launch per step bit for bit.  Lattices the plateau split takes, of
+ * 2^18 sites or more, keep the split for calls of one to three steps.
+ * QLA_KERNEL_TILE = the tile kernel, one launch per step.
  * QLA_KERNEL_MARCH_PLAIN = the marching kernel without the split.
  * Dataflow steps (plateau split, lattices with at least about three work
  * items per resident warp: 16384^2 at 192-row segments, 8192^2 at 64): a
@@ -288,7 +296,8 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * read the sites it stores, have finished step s - 1 (each unit reaches
  * four sites along x and y, Eqs. 2e6 and 2e9); the per-step tail of idle
  * warps goes away and taller segments (fewer recomputed halo rows) pay.
- * Results are bitwise those of one launch per step.  Each wait gives up
+ * Results are bitwise those of one launch per step.
+ * Each wait of a dataflow or resident-tile launch gives up
  * after about two seconds of SM cycles; the next synchronising read
  * (qla_energy, qla_energy_box, qla_divergence, qla_probe, qla_fields,
  * qla_get_state) then returns QLA_ETIMEOUT and the state is undefined until
@@ -331,7 +340,9 @@ qla_status qla_flow_item_deps(int nx, int ny, int segment_rows, int item, int *d
  * handed out at that position of each dataflow launch (step-major: step s,
  * unit k at s * units + k) finish without counting itself, so the units
  * that depend on it wait out their limit and the next synchronising read
- * returns QLA_ETIMEOUT with no fault; -1 restores normal. */
+ * returns QLA_ETIMEOUT with no fault; -1 restores normal.  Resident-tile
+ * launches take the same two settings, their position being step s, tile t
+ * at s * tiles + t. */
 qla_status qla_debug_flow(qla_ctx *ctx, long long budget_cycles, long long withhold_unit);
 
 /* Energy of caller-owned device planes, allocating nothing.

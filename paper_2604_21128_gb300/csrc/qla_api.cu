@@ -21,6 +21,11 @@ static bool march_ok(const qla_ctx *c) {
     return march_supported(c) && offsets32_ok(size_t(c->P), c->plane_elems);
 }
 
+cudaError_t reset_wait_flag(qla_ctx *c) {
+    return c->flow_unchecked ? cudaSuccess
+                             : cudaMemsetAsync(c->wait_flag, 0, sizeof(int), c->stream);
+}
+
 Layout layout_for(int nx, int ny, int prec, unsigned flags) {
     Layout L{};
     const size_t elt = prec == QLA_FP64 ? 8 : 4;
@@ -47,7 +52,10 @@ Layout layout_for(int nx, int ny, int prec, unsigned flags) {
     L.staging = off;  off += align256(sites * 8);
     // partials: up to DIV_TERMS doubles per block (energy uses one)
     L.partials = off; off += align256(nb * 8 * DIV_TERMS);
-    L.result = off;   off += align256(8 * DIV_TERMS);
+    // DIV_TERMS doubles, then the wait flag
+    static_assert(8 * DIV_TERMS <= WAIT_FLAG_OFFSET, "the wait flag follows the results");
+    L.result = off;   off += align256(WAIT_FLAG_OFFSET + sizeof(int));
+    L.tile_done = off; off += align256(TILE_COUNTERS * sizeof(unsigned));
     L.n_x = L.n_y = L.ttable = 0;
     if (flags & QLA_ANISOTROPIC) {
         L.n_x = off; off += align256(L.plane_elems * 8);
@@ -118,16 +126,34 @@ struct DeviceGuard {
 };
 
 // After a synchronisation of the context's stream: QLA_ETIMEOUT if a
-// dataflow step launched since the last check gave up a dependency wait.
-qla_status check_flow(qla_ctx *c, const char *what) {
-    bool t = false;
-    const cudaError_t e = flow_timed_out(c, &t);
-    if (e != cudaSuccess) return cuda_fail(c, e, what);
-    if (t)
+// step launched since the last check gave up a wait.  flag: the wait flag
+// where the call has already copied it, else null.
+qla_status check_flow(qla_ctx *c, const char *what, const int *flag = nullptr) {
+    if (!c->flow_unchecked) return QLA_OK;
+    int v = 0;
+    if (flag) {
+        v = *flag;
+    } else {
+        const cudaError_t e = cudaMemcpy(&v, c->wait_flag, sizeof(int), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(c, e, what);
+    }
+    c->flow_unchecked = false;
+    if (v)
         return fail(c, QLA_ETIMEOUT,
-                    "%s: a dataflow step's dependency wait ran out; the state is undefined "
+                    "%s: a step's wait for its neighbours ran out; the state is undefined "
                     "until it is set again", what);
     return QLA_OK;
+}
+
+// The first n (<= DIV_TERMS) results of a reduction and, in the same copy,
+// the wait flag; synchronises.
+qla_status fetch_results(qla_ctx *c, double *out, int n, const char *what) {
+    struct { double v[WAIT_FLAG_OFFSET / 8]; int flag; } buf;
+    QLA_CUDA(c, cudaMemcpyAsync(&buf, c->result, WAIT_FLAG_OFFSET + sizeof(int),
+                                cudaMemcpyDeviceToHost, c->stream), what);
+    QLA_CUDA(c, cudaStreamSynchronize(c->stream), what);
+    for (int k = 0; k < n; ++k) out[k] = buf.v[k];
+    return check_flow(c, what, &buf.flag);
 }
 
 qla_status usable(qla_ctx *c) {
@@ -219,6 +245,8 @@ qla_status qla_init_grid(qla_ctx **out, int nx, int ny, double delta, int precis
     c->staging = reinterpret_cast<double *>(c->ws + L.staging);
     c->partials = reinterpret_cast<double *>(c->ws + L.partials);
     c->result = reinterpret_cast<double *>(c->ws + L.result);
+    c->wait_flag = reinterpret_cast<int *>(c->ws + L.result + WAIT_FLAG_OFFSET);
+    c->tile_done = reinterpret_cast<unsigned *>(c->ws + L.tile_done);
     c->energy_blocks = L.energy_blocks;
     c->tensor = (flags & QLA_ANISOTROPIC) != 0;
     if (c->tensor) {
@@ -411,13 +439,7 @@ qla_status qla_energy_box(qla_ctx *c, int i0, int j0, int w, int h, double *out)
     DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, QLA_ECUDA, "qla_energy_box: cannot select device");
     QLA_CUDA(c, launch_energy_box(c, i0, j0, w, h), "qla_energy_box: kernel");
-    QLA_CUDA(c, cudaMemcpyAsync(out, c->result, 8, cudaMemcpyDeviceToHost, c->stream),
-             "qla_energy_box: copy");
-    QLA_CUDA(c, cudaStreamSynchronize(c->stream), "qla_energy_box: sync");
-    {
-        const qla_status f = check_flow(c, "qla_energy_box");
-        if (f != QLA_OK) return f;
-    }
+    if ((s = fetch_results(c, out, 1, "qla_energy_box")) != QLA_OK) return s;
     if (!std::isfinite(*out)) return fail(c, QLA_ENONFINITE, "qla_energy_box: energy is %g", *out);
     return QLA_OK;
 }
@@ -488,13 +510,23 @@ qla_status qla_step(qla_ctx *c, long long n_steps) {
         return fail(c, QLA_ESTATE, "qla_step: set a medium and a state first");
     DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, QLA_ECUDA, "qla_step: cannot select device");
-    if ((c->tensor && c->P == 6) || c->vmode == V_LCU) {
-        // the tile kernel with this step's V applied in the same launch:
-        // every pair with its own angle, or the LCU branches
+    // V applied by the step that computes it (tensor media, the LCU branches)
+    // rather than by the next one
+    const bool v_now = (c->tensor && c->P == 6) || c->vmode == V_LCU;
+    if (c->step_kernel == QLA_KERNEL_AUTO && !c->dstable) {
+        // small lattices: every tile resident, many steps per launch
+        for (long long k = 0; n_steps > 0; n_steps -= k) {
+            QLA_CUDA(c, launch_steps_resident(c, n_steps, &k), "qla_step: resident tiles");
+            if (k == 0) break;
+            c->launches++;
+            c->cur ^= int(k & 1);
+            c->pending_v = !v_now && c->vmode != V_NONE;
+        }
+        if (n_steps == 0) return QLA_OK;
+    }
+    if (v_now) {
         for (long long k = 0; k < n_steps; ++k) {
-            QLA_CUDA(c, c->tensor && c->P == 6
-                            ? launch_step_tensor(c, c->state[c->cur], c->state[c->cur ^ 1])
-                            : launch_step_tile(c, c->state[c->cur], c->state[c->cur ^ 1], false),
+            QLA_CUDA(c, launch_step_tile(c, c->state[c->cur], c->state[c->cur ^ 1], false),
                      "qla_step: kernel");
             c->launches++;
             c->cur ^= 1;
@@ -522,7 +554,7 @@ qla_status qla_step(qla_ctx *c, long long n_steps) {
                        c->step_kernel == QLA_KERNEL_MARCH_PLAIN ||
                        c->step_kernel == QLA_KERNEL_MARCH_STEP ||
                        c->step_kernel == QLA_KERNEL_MARCH_FLOW ||
-                       (c->step_kernel == QLA_KERNEL_AUTO && march_ok(c));
+                       (c->step_kernel == QLA_KERNEL_AUTO && march_ok(c) && !tile_steps_pay(c));
     if (march) {
         // all n steps in persistent dataflow launches where the context
         // takes them
@@ -550,13 +582,7 @@ qla_status qla_energy(qla_ctx *c, double *out) {
     DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, QLA_ECUDA, "qla_energy: cannot select device");
     QLA_CUDA(c, launch_energy(c), "qla_energy: kernel");
-    QLA_CUDA(c, cudaMemcpyAsync(out, c->result, 8, cudaMemcpyDeviceToHost, c->stream),
-             "qla_energy: copy");
-    QLA_CUDA(c, cudaStreamSynchronize(c->stream), "qla_energy: sync");
-    {
-        const qla_status f = check_flow(c, "qla_energy");
-        if (f != QLA_OK) return f;
-    }
+    if ((s = fetch_results(c, out, 1, "qla_energy")) != QLA_OK) return s;
     if (!std::isfinite(*out)) return fail(c, QLA_ENONFINITE, "qla_energy: energy is %g", *out);
     return QLA_OK;
 }
@@ -570,13 +596,7 @@ qla_status qla_divergence(qla_ctx *c, double *out) {
     DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, QLA_ECUDA, "qla_divergence: cannot select device");
     QLA_CUDA(c, launch_divergence(c), "qla_divergence: kernel");
-    QLA_CUDA(c, cudaMemcpyAsync(out, c->result, 8 * DIV_TERMS, cudaMemcpyDeviceToHost, c->stream),
-             "qla_divergence: copy");
-    QLA_CUDA(c, cudaStreamSynchronize(c->stream), "qla_divergence: sync");
-    {
-        const qla_status f = check_flow(c, "qla_divergence");
-        if (f != QLA_OK) return f;
-    }
+    if ((s = fetch_results(c, out, DIV_TERMS, "qla_divergence")) != QLA_OK) return s;
     for (int k = 0; k < DIV_TERMS; ++k)
         if (!std::isfinite(out[k]))
             return fail(c, QLA_ENONFINITE, "qla_divergence: term %d is %g", k, out[k]);

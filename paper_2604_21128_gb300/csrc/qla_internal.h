@@ -401,9 +401,14 @@ struct qla_ctx {
         int n_wx = 0, shift = 0;
         size_t off_xdep = 0, off_ydep = 0, off_ctr = 0;
     } uplan;
-    // dataflow steps: a launch whose wait flag has not been read yet, each
-    // wait's limit in SM cycles, and a test hook (the handed-out unit index
-    // whose completion is withheld, -1 none)
+    // device flag that a wait between tiles or units of steps raises when it
+    // runs out (behind the reduction results, so one copy brings both), and
+    // the resident tile steps' counters
+    int *wait_flag = nullptr;
+    unsigned *tile_done = nullptr;
+    // launches that wait on one another's tiles or units: one whose wait flag
+    // has not been read yet, each wait's limit in SM cycles, and a test hook
+    // (the handed-out unit index whose completion is withheld, -1 none)
     bool flow_unchecked = false;
     long long flow_budget = 1LL << 32;
     long long flow_withhold = -1;
@@ -412,10 +417,16 @@ struct qla_ctx {
 };
 
 namespace qla {
+// Byte offset of the wait flag in the result region, and the counters held
+// for resident tile steps (more tiles than any GPU holds at once).
+constexpr size_t WAIT_FLAG_OFFSET = 64;
+constexpr int TILE_COUNTERS = 2048;
+
 // Workspace layout: offsets of each region (bytes, 256-aligned).
 struct Layout {
     size_t state[2], midx, table, keys, counter, n, staging, partials, result, total;
     size_t n_x, n_y, ttable;  // QLA_ANISOTROPIC only (else 0)
+    size_t tile_done;         // TILE_COUNTERS counters
     size_t dstable;           // QLA_DOUBLE_SINGLE only (else 0)
     size_t items, items_cap;  // FP32 E_z only (else 0): marching work-item list
     size_t plane_elems;
@@ -439,7 +450,6 @@ cudaError_t raw_to_f64(int prec, const void *state, size_t plane_elems, int comp
 cudaError_t raw_energy(int prec, const void *state, size_t plane_elems, int nx, int rows,
                        int pitch, double *partials, int nblocks, double *result, cudaStream_t st);
 cudaError_t launch_medium_tensor(qla_ctx *c);
-cudaError_t launch_step_tensor(qla_ctx *c, const void *in, void *out);
 // QLA_DOUBLE_SINGLE: the marching step on word-pair state with the
 // double-single records, and the in-place conversions of the state buffer
 // between FP64 and word pairs.
@@ -476,9 +486,15 @@ cudaError_t launch_step_march(qla_ctx *c, const void *in, void *out, bool vin);
 // 1)].  *done = false (nothing enqueued) where the context does not take
 // them; needs a pending potential step if the context has a potential.
 cudaError_t launch_step_flow(qla_ctx *c, long long n_steps, bool *done);
-// Reads (and clears) the wait flag of the dataflow launches since the last
-// read; the stream must be idle.  Returns true if a wait ran out.
-cudaError_t flow_timed_out(qla_ctx *c, bool *timed_out);
+// The steps of a lattice whose tiles are all resident at once, in one launch
+// from c->state[c->cur] with c->pending_v; *done steps were enqueued (0 where
+// the lattice has too many tiles), the result in state[c->cur ^ (*done & 1)].
+cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done);
+// Whether an automatic context's steps go to the tile kernel although the
+// marching kernel takes its lattice.
+bool tile_steps_pay(const qla_ctx *c);
+// Clears the wait flag unless launches since its last read may have raised it.
+cudaError_t reset_wait_flag(qla_ctx *c);
 bool march_supported(const qla_ctx *c);
 int march_lane_cols(const qla_ctx *c);
 }  // namespace qla

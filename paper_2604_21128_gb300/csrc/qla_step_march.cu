@@ -317,8 +317,7 @@ cudaError_t build_plateau_plan(qla_ctx *c, int seg, bool flow) {
         off_ydep = off_xdep + (xd.size() * 4 + 15) / 16 * 16;
         off_ctr = off_ydep + (yd.size() * 4 + 15) / 16 * 16;
         const size_t end = off_ctr + 16 + size_t(n_items) * 4;
-        // the wait flag sits in the last 16 bytes of the region
-        if (!ok_x || !ok_y || end + 16 > c->items_cap * sizeof(int4)) return cudaSuccess;
+        if (!ok_x || !ok_y || end > c->items_cap * sizeof(int4)) return cudaSuccess;
         blob.resize(off_ctr, 0);
         memcpy(blob.data() + off_xdep, xd.data(), xd.size() * 4);
         memcpy(blob.data() + off_ydep, yd.data(), yd.size() * 4);
@@ -391,12 +390,6 @@ cudaError_t build_plateau_plan_ds(qla_ctx *c, int seg) {
     return cudaSuccess;
 }
 
-// The dataflow launches' wait flag: the last 16 bytes of the unit region,
-// which no plan uses, so it survives plan rebuilds until the host reads it.
-int *flow_flag(qla_ctx *c) {
-    return reinterpret_cast<int *>(reinterpret_cast<char *>(c->items) + c->items_cap * 16 - 16);
-}
-
 // The plan of segments of `seg` rows (dataflow order and tables with
 // `flow`), built unless it is the current one.  A dataflow plan that does
 // not fit the workspace falls back to the per-step plan of the same
@@ -462,9 +455,9 @@ cudaError_t launch_flow(qla_ctx *c, const void *in, void *out, long long n_steps
     const auto &u = c->uplan;
     char *base = reinterpret_cast<char *>(c->items);
     unsigned *ctr = reinterpret_cast<unsigned *>(base + u.off_ctr);
-    int *err = flow_flag(c);
-    if (!c->flow_unchecked) {
-        const cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), c->stream);
+    int *err = c->wait_flag;
+    {
+        const cudaError_t e = reset_wait_flag(c);
         if (e != cudaSuccess) return e;
     }
     // units x steps of one launch below 2^31, item counters below 2^32
@@ -718,17 +711,6 @@ cudaError_t launch_step_flow(qla_ctx *c, long long n_steps, bool *done) {
     if (e != cudaSuccess) return e;
     if (n_steps & 1) c->cur ^= 1;
     c->pending_v = c->vmode != V_NONE;
-    return cudaSuccess;
-}
-
-cudaError_t flow_timed_out(qla_ctx *c, bool *timed_out) {
-    *timed_out = false;
-    if (!c->flow_unchecked) return cudaSuccess;
-    int v = 0;
-    const cudaError_t e = cudaMemcpy(&v, flow_flag(c), sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return e;
-    c->flow_unchecked = false;
-    *timed_out = v != 0;
     return cudaSuccess;
 }
 

@@ -1,0 +1,81 @@
+"""Resident-tile launches (all steps of a qla_step call on a small lattice in
+one launch of the tile kernel, tiles waiting for their neighbours) against one
+tile launch per step: the same bits at the edges of the tile sizes, for every
+potential reading and medium, and a wait that runs out is reported."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2604_21128_gb300 import inputs, qla
+
+pytestmark = pytest.mark.gpu
+
+# one tile, one tile and a site, tiles of 12 and 13, long and thin, many tiles
+SHAPES = [(5, 7), (24, 24), (25, 24), (47, 49), (130, 9), (33, 260), (256, 251)]
+
+
+def run(shape, kernel, calls, precision="fp32", te=True, potential="rotation", tensor=False):
+    nx, ny = shape
+    n = inputs.random_medium(nx, ny, seed=nx + 7 * ny, lo=1.0, hi=2.5)
+    n[: ny // 2] = 2.0                      # shared records next to own ones
+    with qla.Grid(nx, ny, 1.0, precision, te_only=te, potential=potential, tensor=tensor) as g:
+        g.set_step_kernel(kernel)
+        g.set_medium(np.stack([n, 1.1 * n, 1.2 * n]) if tensor else n)
+        g.set_state(inputs.random_state(nx, ny, seed=nx, planes=3 if te else 6))
+        before = g.launches
+        for k in calls:
+            g.step(k)
+        return g.launches - before, g.get_state(), g.energy()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("te", [True, False])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_resident_tiles_agree_bitwise(shape, te, precision):
+    a = run(shape, "auto", (4, 1, 6), precision, te)
+    b = run(shape, "tile", (11,), precision, te)
+    assert a[0] == 3 and b[0] == 11
+    assert np.array_equal(a[1], b[1]) and a[2] == b[2]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("kw", [dict(potential="literal"), dict(potential="none"),
+                                dict(potential="lcu"), dict(te=False, potential="lcu"),
+                                dict(te=False, tensor=True),
+                                dict(te=False, tensor=True, potential="lcu")])
+def test_resident_tiles_of_every_reading(kw, precision):
+    a = run((61, 50), "auto", (5,), precision, **kw)
+    b = run((61, 50), "tile", (5,), precision, **kw)
+    assert a[0] == 1 and b[0] == 5
+    assert np.array_equal(a[1], b[1]) and a[2] == b[2]
+
+
+def test_tile_wait_runs_out_without_fault():
+    """A tile that does not publish a step: its neighbours wait out a short
+    limit, every CTA leaves, the next read returns QLA_ETIMEOUT, and with the
+    state set again the context steps exactly as before."""
+    nx, ny = 96, 72
+    n = inputs.random_medium(nx, ny, seed=3)
+    q0 = inputs.random_state(nx, ny, seed=4)
+    out = []
+    with qla.Grid(nx, ny, 1.0, "fp64") as g:
+        g.set_medium(n)
+        for withhold in (3, -1):
+            g.set_state(q0)
+            g.debug_flow(budget_cycles=2_000_000 if withhold >= 0 else 0, withhold_unit=withhold)
+            t0 = time.perf_counter()
+            g.step(6)
+            if withhold >= 0:
+                with pytest.raises(qla.QLAError) as e:
+                    g.energy()
+                assert e.value.status == 5     # QLA_ETIMEOUT
+                assert time.perf_counter() - t0 < 30.0
+        out.append(g.get_state())
+    with qla.Grid(nx, ny, 1.0, "fp64") as g:
+        g.set_step_kernel("tile")
+        g.set_medium(n)
+        g.set_state(q0)
+        g.step(6)
+        out.append(g.get_state())
+    assert np.array_equal(out[0], out[1])

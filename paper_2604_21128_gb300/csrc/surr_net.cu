@@ -30,7 +30,7 @@ namespace {
 
 constexpr int LEVELS = 5;
 constexpr int WIDTH[LEVELS] = {32, 64, 128, 256, 256};
-constexpr int FEAT = 6, NOUT = 3, CPAD = 32;
+constexpr int FEAT = 6, NOUT = 3, CPAD = 16;   // inputs and outputs padded to one K step
 constexpr int NCONV = 10;
 
 struct ConvSpec {
@@ -63,21 +63,22 @@ struct surr_net {
     int H = 0, W = 0, maxB = 0;
     cudaStream_t stream = nullptr;
     char *mem = nullptr;
-    // parameters
-    float *wf[NCONV], *bias[NCONV];           // master
-    float *gw[NCONV], *gb[NCONV];             // gradients
-    float *mw[NCONV], *vw[NCONV], *mb[NCONV], *vb[NCONV];
-    bf16 *wb[NCONV], *wt[NCONV];              // bf16 copy, flipped-transposed copy
+    // parameters, gradients, Adam state and the BF16 copies, by layer
+    NetParams prm;
     size_t nw[NCONV];
-    // activations (bf16), per level: E, D (l < 4), P (l >= 1), U (l < 4)
+    // activations (blocked BF16), per level: E, D (l < 4), and the inputs of
+    // the convolutions, P = pool E (l >= 1), U = up D (l < 4)
     bf16 *X, *E[LEVELS], *D[LEVELS], *Pl[LEVELS], *U[LEVELS];
-    float *Y;                                  // [P0][CPAD]
-    // gradients (fp32)
-    float *dY, *dE[LEVELS], *dD[LEVELS], *dP[LEVELS], *dU[LEVELS];
-    bf16 *dz;                                  // scratch
-    float *part, *bpart;
-    double *lpart;
-    int lblocks = 0, bblocks = 0;
+    float *Y;                                  // [P0][NOUT]
+    // gradients (blocked FP32): of D0, of E through the skips, of P and U
+    float *dD0, *dE[LEVELS], *dP[LEVELS], *dU[LEVELS];
+    bf16 *dz, *dz9;                            // of a layer, of the output layer
+    float *part[NCONV], *bpart[NCONV];         // split sums of weights and biases
+    double *lpart;                             // loss partials
+    double *lout;                              // loss and wait flag
+    double *lhost = nullptr;                   // the same, pinned
+    cudaEvent_t ldone = nullptr;
+    int *flag = nullptr;                       // the convolutions' wait flag
     long long step = 0;
     std::string err;
 };
@@ -101,103 +102,62 @@ qla_status nfail(surr_net *n, qla_status s, const char *fmt, ...) {
             return nfail((n), QLA_ECUDA, "%s: %s", (what), cudaGetErrorString(e_)); \
     } while (0)
 
-long long pixels(const surr_net *n, int B, int level) {
-    return (long long)B * (n->H >> level) * (n->W >> level);
-}
-
-// Pixel splits of the weight gradient: one per 4096 pixels, at most 128
-// (at 256^2 x 8 a cap of 32 left the level-0 gradient with too few CTAs:
-// 4.85 ms per training step, 4.54 ms with 128).
-int splits_for(long long P) {
-    long long s = P / 4096;
-    return int(std::max<long long>(1, std::min<long long>(128, s)));
-}
-
-size_t net_bytes(int H, int W, int B, bool with_mem, char **out_mem) {
-    // Two passes: measure with a null base, then carve for real.
-    (void)with_mem;
-    (void)out_mem;
-    size_t total = 0;
-    auto add = [&](size_t bytes) { total += (bytes + 255) & ~size_t(255); };
-    for (int i = 0; i < NCONV; ++i) {
-        const ConvSpec s = spec(i);
-        const size_t nw = size_t(s.cout) * 9 * s.cin;
-        add(nw * 4 * 4);        // master, grad, m, v
-        add(size_t(s.cout) * 4 * 4);
-        add(nw * 2 * 2);        // bf16 copy + flipped copy
-    }
-    const long long P0 = (long long)B * H * W;
-    add(P0 * CPAD * 2);                                    // X
-    for (int l = 0; l < LEVELS; ++l) {
-        const long long Pl = P0 >> (2 * l);
-        add(Pl * WIDTH[l] * 2);                            // E
-        if (l < 4) add(Pl * WIDTH[l] * 2);                 // D
-        if (l >= 1) add(Pl * WIDTH[l - 1] * 2);            // P (input of E_l)
-        if (l < 4) add(Pl * WIDTH[l + 1] * 2);             // U (input of D_l)
-        add(Pl * WIDTH[l] * 4);                            // dE
-        if (l < 4) add(Pl * WIDTH[l] * 4);                 // dD
-        if (l >= 1) add(Pl * WIDTH[l - 1] * 4);            // dP
-        if (l < 4) add(Pl * WIDTH[l + 1] * 4);             // dU
-    }
-    add(P0 * CPAD * 4 * 2);                                // Y, dY
-    add(P0 * 256 * 2);                                     // dz scratch (>= any P_l * C_l)
-    size_t part = 0;
-    for (int i = 0; i < NCONV; ++i) {
-        const ConvSpec s = spec(i);
-        const long long Pin = P0 >> (2 * s.level);
-        part = std::max(part, size_t(splits_for(Pin)) * s.cout * 9 * s.cin);
-    }
-    add(part * 4);
-    add(1024 * 256 * 4);                                   // bias partials
-    add(4096 * 8);                                         // loss partials
-    return total;
-}
-
-void carve_all(surr_net *n, int B) {
+// Lays the network out from n->mem (null: only measured); returns the bytes.
+size_t carve_all(surr_net *n) {
     char *p = n->mem;
+    const int B = n->maxB, H = n->H, W = n->W;
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
+        LayerParams &l = n->prm.l[i];
         const size_t nw = size_t(s.cout) * 9 * s.cin;
         n->nw[i] = nw;
-        n->wf[i] = carve<float>(p, nw);
-        n->gw[i] = carve<float>(p, nw);
-        n->mw[i] = carve<float>(p, nw);
-        n->vw[i] = carve<float>(p, nw);
-        n->bias[i] = carve<float>(p, s.cout);
-        n->gb[i] = carve<float>(p, s.cout);
-        n->mb[i] = carve<float>(p, s.cout);
-        n->vb[i] = carve<float>(p, s.cout);
-        n->wb[i] = carve<bf16>(p, nw);
-        n->wt[i] = carve<bf16>(p, nw);
+        l.cout = s.cout;
+        l.cin = s.cin;
+        l.w = carve<float>(p, nw);
+        l.gw = carve<float>(p, nw);
+        l.mw = carve<float>(p, nw);
+        l.vw = carve<float>(p, nw);
+        l.b = carve<float>(p, s.cout);
+        l.gb = carve<float>(p, s.cout);
+        l.mb = carve<float>(p, s.cout);
+        l.vb = carve<float>(p, s.cout);
+        l.wb = carve<bf16>(p, nw);
+        l.wt = carve<bf16>(p, nw);
     }
-    const long long P0 = (long long)B * n->H * n->W;
-    n->X = carve<bf16>(p, P0 * CPAD);
+    auto act = [&](int c, int l) { return carve<bf16>(p, blocked_elems(B, c, H >> l, W >> l)); };
+    auto grad = [&](int c, int l) {
+        return carve<float>(p, size_t(B) * c * size_t(H >> l) * size_t(W >> l));
+    };
+    size_t dz = 0;
+    n->X = act(CPAD, 0);
     for (int l = 0; l < LEVELS; ++l) {
-        const long long Pl = P0 >> (2 * l);
-        n->E[l] = carve<bf16>(p, Pl * WIDTH[l]);
-        n->D[l] = l < 4 ? carve<bf16>(p, Pl * WIDTH[l]) : nullptr;
-        n->Pl[l] = l >= 1 ? carve<bf16>(p, Pl * WIDTH[l - 1]) : nullptr;
-        n->U[l] = l < 4 ? carve<bf16>(p, Pl * WIDTH[l + 1]) : nullptr;
-        n->dE[l] = carve<float>(p, Pl * WIDTH[l]);
-        n->dD[l] = l < 4 ? carve<float>(p, Pl * WIDTH[l]) : nullptr;
-        n->dP[l] = l >= 1 ? carve<float>(p, Pl * WIDTH[l - 1]) : nullptr;
-        n->dU[l] = l < 4 ? carve<float>(p, Pl * WIDTH[l + 1]) : nullptr;
+        n->E[l] = act(WIDTH[l], l);
+        n->D[l] = l < 4 ? act(WIDTH[l], l) : nullptr;
+        n->Pl[l] = l >= 1 ? act(WIDTH[l - 1], l) : nullptr;
+        n->U[l] = l < 4 ? act(WIDTH[l + 1], l) : nullptr;
+        n->dE[l] = l < 4 ? grad(WIDTH[l], l) : nullptr;
+        n->dP[l] = l >= 1 ? grad(WIDTH[l - 1], l) : nullptr;
+        n->dU[l] = l < 4 ? grad(WIDTH[l + 1], l) : nullptr;
+        dz = std::max(dz, blocked_elems(B, WIDTH[l], H >> l, W >> l));
     }
-    n->Y = carve<float>(p, P0 * CPAD);
-    n->dY = carve<float>(p, P0 * CPAD);
-    n->dz = carve<bf16>(p, P0 * 256);
-    size_t part = 0;
+    n->dD0 = grad(WIDTH[0], 0);
+    n->Y = carve<float>(p, size_t(B) * H * W * NOUT);
+    n->dz = carve<bf16>(p, dz);
+    n->dz9 = act(CPAD, 0);
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
-        const long long Pin = P0 >> (2 * s.level);
-        part = std::max(part, size_t(splits_for(Pin)) * s.cout * 9 * s.cin);
+        const int h = H >> s.level, w = W >> s.level;
+        // smaller batches never take more splits or chunks
+        n->part[i] = carve<float>(p, size_t(weight_grad_splits(B, h, w)) * n->nw[i]);
+        n->bpart[i] = carve<float>(p, size_t(bias_blocks(B, h, w)) * s.cout);
     }
-    n->part = carve<float>(p, part);
-    n->bpart = carve<float>(p, 1024 * 256);
-    n->lpart = carve<double>(p, 4096);
+    // the lattice checks of surr_advance use 768 doubles of it
+    n->lpart = carve<double>(p, size_t(std::max(768, bias_blocks(B, H, W))));
+    n->lout = carve<double>(p, 2);
+    return size_t(p - n->mem);
 }
 
-// conv layer i: its input tensor for batch B
+// conv layer i: its input and output tensors
 const bf16 *conv_input(const surr_net *n, int i) {
     if (i == 0) return n->X;
     if (i < 5) return n->Pl[i];
@@ -211,97 +171,91 @@ bf16 *conv_output(surr_net *n, int i) {
     return nullptr;
 }
 
-qla_status forward(surr_net *n, int B) {
-    cudaStream_t st = n->stream;
+// Ten launches: each convolution writes its output and, where the next layer
+// reads it pooled (encoder) or upsampled (decoder), that too.
+qla_status forward(surr_net *n, int B, float *y) {
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
         const int l = s.level;
-        const int h = n->H >> l, w = n->W >> l;
-        // inputs: pool before encoder levels >= 1, upsample before decoder
-        if (i >= 1 && i < 5) {
-            const long long m = pixels(n, B, l) * WIDTH[l - 1];
-            k_pool<<<ew_blocks(m / 8), 256, 0, st>>>(n->E[l - 1], B, h * 2, w * 2, WIDTH[l - 1],
-                                                 n->Pl[l]);
-        } else if (i >= 5 && i < 9) {
-            const bf16 *src = (i == 5) ? n->E[4] : n->D[l + 1];
-            const long long m = pixels(n, B, l) * WIDTH[l + 1];
-            k_up<<<ew_blocks(m / 8), 256, 0, st>>>(src, B, h / 2, w / 2, WIDTH[l + 1], n->U[l]);
-        }
-        NCUDA(n, cudaGetLastError(), "surrogate: resample");
-        ConvArgs a{conv_input(n, i), B, h, w, s.cin, n->wb[i], s.cout, n->bias[i],
-                   s.skip ? n->E[l] : nullptr, conv_output(n, i), n->Y};
-        NCUDA(n, conv3x3(a, i == 9 ? OUT_F32 : OUT_BF16, s.act, s.skip, st), "surrogate: conv");
+        ConvArgs a{};
+        a.in = conv_input(n, i);
+        a.B = B;
+        a.H = n->H >> l;
+        a.W = n->W >> l;
+        a.cin = s.cin;
+        a.cout = s.cout;
+        a.w = n->prm.l[i].wb;
+        a.bias = n->prm.l[i].b;
+        a.skip = s.skip ? n->E[l] : nullptr;
+        a.out = conv_output(n, i);
+        a.pool = i < 4 ? n->Pl[l + 1] : nullptr;
+        a.up = i >= 4 && i < 8 ? n->U[l - 1] : nullptr;
+        a.out_f = y;
+        a.n_out = NOUT;
+        NCUDA(n, conv3x3(a, i == 9 ? EP_OUT : EP_ACT, n->stream), "surrogate: conv");
     }
     return QLA_OK;
 }
 
-// Backward through conv layer i given dOut (fp32) of its output.  Writes
-// the weight and bias gradients, adds the pre-activation gradient to the
-// skip tensor's gradient, and returns the input gradient in dIn (fp32,
-// overwritten).
-qla_status conv_backward(surr_net *n, int i, int B, const float *dOut, float *dSkip, float *dIn) {
-    cudaStream_t st = n->stream;
+// The weight gradient's split sums of layer i from its dz, and (d_in) the
+// gradient of its input.
+qla_status conv_backward(surr_net *n, int i, int B, const bf16 *dz, float *d_in, SumJobs &jobs,
+                         int &njobs) {
     const ConvSpec s = spec(i);
-    const int l = s.level, h = n->H >> l, w = n->W >> l;
-    const long long P = pixels(n, B, l);
-    const int blocks = int(std::min<long long>(1024, std::max<long long>(1, P / 256)));
-    NCUDA(n, act_back(dOut, conv_output(n, i), P, s.cout, s.act, n->dz, dSkip, n->bpart, blocks, st),
-          "surrogate: activation backward");
-    NCUDA(n, sum_splits(n->bpart, blocks, s.cout, n->gb[i], st), "surrogate: bias grad");
-    const int splits = splits_for(P);
-    NCUDA(n, weight_grad(n->dz, conv_input(n, i), B, h, w, s.cout, s.cin, splits, n->part, st),
+    const int h = n->H >> s.level, w = n->W >> s.level;
+    const LayerParams &l = n->prm.l[i];
+    const int splits = weight_grad_splits(B, h, w);
+    NCUDA(n, weight_grad(dz, conv_input(n, i), B, h, w, s.cout, s.cin, splits, n->part[i],
+                         n->stream),
           "surrogate: weight grad");
-    NCUDA(n, sum_splits(n->part, splits, (long long)s.cout * 9 * s.cin, n->gw[i], st),
-          "surrogate: weight grad sum");
-    if (dIn) {
-        NCUDA(n, cudaMemsetAsync(dIn, 0, sizeof(float) * P * s.cin, st), "surrogate: clear");
-        ConvArgs a{n->dz, B, h, w, s.cout, n->wt[i], s.cin, nullptr, nullptr, nullptr, dIn};
-        NCUDA(n, conv3x3(a, ACC_F32, false, false, st), "surrogate: input grad");
+    jobs.j[njobs++] = {n->part[i], l.gw, splits, (long long)n->nw[i], false};
+    jobs.j[njobs++] = {n->bpart[i], l.gb, bias_blocks(B, h, w), s.cout, false};
+    if (d_in) {
+        ConvArgs a{};
+        a.in = dz;
+        a.B = B;
+        a.H = h;
+        a.W = w;
+        a.cin = s.cout;
+        a.cout = s.cin;
+        a.w = l.wt;
+        a.out_f = d_in;
+        NCUDA(n, conv3x3(a, EP_F32, n->stream), "surrogate: input grad");
     }
     return QLA_OK;
 }
 
 qla_status backward(surr_net *n, int B) {
-    cudaStream_t st = n->stream;
-    for (int i = 0; i < NCONV; ++i) {
-        const ConvSpec s = spec(i);
-        k_flip<<<ew_blocks(n->nw[i]), 256, 0, st>>>(n->wb[i], s.cout, s.cin, n->wt[i]);
-    }
-    NCUDA(n, cudaGetLastError(), "surrogate: flip");
-    for (int l = 0; l < LEVELS; ++l) {
-        NCUDA(n, cudaMemsetAsync(n->dE[l], 0, sizeof(float) * pixels(n, B, l) * WIDTH[l], st),
-              "surrogate: clear");
-    }
+    SumJobs jobs{};
+    int njobs = 0;
     qla_status r;
-    // output conv: dY -> dD0
-    if ((r = conv_backward(n, 9, B, n->dY, nullptr, n->dD[0])) != QLA_OK) return r;
-    // decoder levels 0..3 (conv i = 8 - l): dD_l -> dU_l, skip into dE_l
+    // through layer i's activation: dz from the gradient of its output
+    auto through = [&](int i, GradSource src, const float *a, const float *b, float *g_out) {
+        const ConvSpec s = spec(i);
+        const ActBack args{a, b, conv_output(n, i), n->dz, g_out, n->bpart[i], B,
+                           n->H >> s.level, n->W >> s.level, s.cout};
+        NCUDA(n, act_back(args, src, n->stream), "surrogate: activation backward");
+        return QLA_OK;
+    };
+    // output convolution (dz9 from the loss) -> dD0
+    if ((r = conv_backward(n, 9, B, n->dz9, n->dD0, jobs, njobs)) != QLA_OK) return r;
+    // decoder levels 0..3 (layer 8 - l): dD_l -> dU_l, the skip's share to dE_l
     for (int l = 0; l < 4; ++l) {
         const int i = 8 - l;
-        if ((r = conv_backward(n, i, B, n->dD[l], n->dE[l], n->dU[l])) != QLA_OK) return r;
-        // up_l came from D_{l+1} (l < 3) or E4 (l = 3)
-        const int h = n->H >> (l + 1), w = n->W >> (l + 1);
-        float *dst = l < 3 ? n->dD[l + 1] : n->dE[4];
-        const long long m = pixels(n, B, l + 1) * WIDTH[l + 1];
-        if (l < 3) {
-            k_up_back<<<ew_blocks(m / 4), 256, 0, st>>>(n->dU[l], B, h, w, WIDTH[l + 1], dst);
-        } else {
-            // dE4 only receives this gradient; D3's up-sampled input is E4
-            k_up_back<<<ew_blocks(m / 4), 256, 0, st>>>(n->dU[l], B, h, w, WIDTH[l + 1], dst);
-        }
-        NCUDA(n, cudaGetLastError(), "surrogate: upsample backward");
+        if ((r = through(i, l == 0 ? G_DIRECT : G_UPSUM, l == 0 ? n->dD0 : n->dU[l - 1], nullptr,
+                         n->dE[l])) != QLA_OK)
+            return r;
+        if ((r = conv_backward(n, i, B, n->dz, n->dU[l], jobs, njobs)) != QLA_OK) return r;
     }
-    // encoder levels 4..0: dE_l -> dP_l -> dE_{l-1} (accumulated)
+    // encoder levels 4..0: dE_l (upsampling; skip and pooling below) -> dP_l
     for (int l = 4; l >= 0; --l) {
-        float *din = l >= 1 ? n->dP[l] : nullptr;
-        if ((r = conv_backward(n, l, B, n->dE[l], nullptr, din)) != QLA_OK) return r;
-        if (l >= 1) {
-            const int H = n->H >> (l - 1), W = n->W >> (l - 1);
-            const long long m = pixels(n, B, l - 1) * WIDTH[l - 1];
-            k_pool_back<<<ew_blocks(m / 4), 256, 0, st>>>(n->dP[l], B, H, W, WIDTH[l - 1], n->dE[l - 1]);
-            NCUDA(n, cudaGetLastError(), "surrogate: pool backward");
-        }
+        if ((r = l == 4 ? through(4, G_UPSUM, n->dU[3], nullptr, nullptr)
+                        : through(l, G_POOL, n->dE[l], n->dP[l + 1], nullptr)) != QLA_OK)
+            return r;
+        if ((r = conv_backward(n, l, B, n->dz, l >= 1 ? n->dP[l] : nullptr, jobs, njobs)) != QLA_OK)
+            return r;
     }
+    NCUDA(n, sum_splits(jobs, njobs, n->stream), "surrogate: gradient sums");
     return QLA_OK;
 }
 
@@ -318,33 +272,49 @@ qla_status tc_waits_ok(surr_net *n) {
     return QLA_OK;
 }
 
-qla_status loss(surr_net *n, int B, const float *target, double *out) {
-    const long long P = pixels(n, B, 0);
-    const int blocks = std::min(n->lblocks, ew_blocks(P));
-    k_mse<<<blocks, 256, 0, n->stream>>>(n->Y, CPAD, target, NOUT, P, n->dY, n->lpart);
-    NCUDA(n, cudaGetLastError(), "surrogate: loss");
-    std::vector<double> h(blocks);
-    NCUDA(n, cudaMemcpyAsync(h.data(), n->lpart, sizeof(double) * blocks, cudaMemcpyDeviceToHost,
-                             n->stream), "surrogate: loss copy");
-    NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
-    const qla_status w = tc_waits_ok(n);
-    if (w != QLA_OK) return w;
-    double s = 0.0;
-    for (double v : h) s += v;
-    *out = s;
+// The loss of n->Y, its gradient into dz9, and loss and wait flag on their
+// way to the host.
+qla_status loss_begin(surr_net *n, int B, const float *target) {
+    NCUDA(n, mse(n->Y, target, NOUT, B, n->H, n->W, CPAD / 8, n->dz9, n->lpart, n->bpart[9],
+                 n->stream), "surrogate: loss");
+    NCUDA(n, loss_final(n->lpart, bias_blocks(B, n->H, n->W), n->flag, n->lout, n->stream),
+          "surrogate: loss sum");
+    NCUDA(n, cudaMemcpyAsync(n->lhost, n->lout, 16, cudaMemcpyDeviceToHost, n->stream),
+          "surrogate: loss copy");
+    NCUDA(n, cudaEventRecord(n->ldone, n->stream), "surrogate: loss event");
+    return QLA_OK;
+}
+
+// Waits for the loss (not for the work enqueued after it).
+qla_status loss_end(surr_net *n, double *out) {
+    NCUDA(n, cudaEventSynchronize(n->ldone), "surrogate: sync");
+    *out = n->lhost[0];
+    if (n->lhost[1] != 0.0) {
+        // the flag is cleared only once nothing of this call reads it any more
+        NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
+        return tc_waits_ok(n);
+    }
     return QLA_OK;
 }
 
 qla_status pack(surr_net *n, const float *feat, int B) {
-    const long long P = pixels(n, B, 0);
-    k_pack_in<<<ew_blocks(P), 256, 0, n->stream>>>(feat, P, FEAT, CPAD, n->X);
-    NCUDA(n, cudaGetLastError(), "surrogate: pack");
+    NCUDA(n, pack_features(feat, B, n->H, n->W, FEAT, CPAD, n->X, n->stream), "surrogate: pack");
     return QLA_OK;
 }
 
 qla_status check_batch(surr_net *n, int B) {
     if (B < 1 || B > n->maxB) return nfail(n, QLA_EINVAL, "batch %d outside 1..%d", B, n->maxB);
     return QLA_OK;
+}
+
+// Forward, loss and backward enqueued.
+qla_status enqueue_grad(surr_net *n, const float *feat, const float *target, int B) {
+    qla_status s = check_batch(n, B);
+    if (s != QLA_OK) return s;
+    if ((s = pack(n, feat, B)) != QLA_OK) return s;
+    if ((s = forward(n, B, n->Y)) != QLA_OK) return s;
+    if ((s = loss_begin(n, B, target)) != QLA_OK) return s;
+    return backward(n, B);
 }
 
 }  // namespace
@@ -455,7 +425,11 @@ size_t surr_workspace_bytes(int height, int width, int max_batch) {
     if (height < 16 || width < 16 || height % 16 || width % 16 || max_batch < 1) return 0;
     // the elementwise kernels index the widest level-0 tensor with 32 bits
     if ((long long)max_batch * height * width * 32 >= (1LL << 31)) return 0;
-    return net_bytes(height, width, max_batch, false, nullptr);
+    surr_net n;
+    n.H = height;
+    n.W = width;
+    n.maxB = max_batch;
+    return carve_all(&n);
 }
 
 qla_status surr_create(surr_net **out, int height, int width, int max_batch,
@@ -474,12 +448,22 @@ qla_status surr_create(surr_net **out, int height, int width, int max_batch,
     n->maxB = max_batch;
     n->stream = static_cast<cudaStream_t>(cuda_stream);
     n->mem = static_cast<char *>(workspace);
-    carve_all(n, max_batch);
-    n->lblocks = 4096;
+    carve_all(n);
+    // the output layer's dz keeps zeros in its padded channels
+    if (conv_tc_error_ptr(&n->flag) != cudaSuccess ||
+        cudaMallocHost(&n->lhost, 16) != cudaSuccess ||
+        cudaEventCreateWithFlags(&n->ldone, cudaEventDisableTiming) != cudaSuccess ||
+        cudaMemsetAsync(n->dz9, 0, blocked_elems(max_batch, CPAD, height, width) * 2,
+                        n->stream) != cudaSuccess) {
+        cudaGetLastError();
+        surr_destroy(n);
+        return QLA_ECUDA;
+    }
     // He-style initialisation from a seeded generator (host), zero biases
     std::mt19937_64 rng(seed);
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
+        LayerParams &l = n->prm.l[i];
         std::vector<float> w(n->nw[i], 0.f);
         const double fan_in = 9.0 * s.cin_real;
         std::normal_distribution<double> nd(0.0, std::sqrt(2.0 / fan_in) * (i == 9 ? 0.1 : 1.0));
@@ -487,21 +471,20 @@ qla_status surr_create(surr_net **out, int height, int width, int max_batch,
             for (int t = 0; t < 9; ++t)
                 for (int ci = 0; ci < s.cin_real; ++ci)
                     w[(size_t(co) * 9 + t) * s.cin + ci] = float(nd(rng));
-        std::vector<float> zeros(s.cout, 0.f);
-        if (cudaMemcpyAsync(n->wf[i], w.data(), n->nw[i] * 4, cudaMemcpyHostToDevice, n->stream) ||
-            cudaMemsetAsync(n->bias[i], 0, s.cout * 4, n->stream) ||
-            cudaMemsetAsync(n->mw[i], 0, n->nw[i] * 4, n->stream) ||
-            cudaMemsetAsync(n->vw[i], 0, n->nw[i] * 4, n->stream) ||
-            cudaMemsetAsync(n->mb[i], 0, s.cout * 4, n->stream) ||
-            cudaMemsetAsync(n->vb[i], 0, s.cout * 4, n->stream) ||
+        if (cudaMemcpyAsync(l.w, w.data(), n->nw[i] * 4, cudaMemcpyHostToDevice, n->stream) ||
+            cudaMemsetAsync(l.b, 0, s.cout * 4, n->stream) ||
+            cudaMemsetAsync(l.mw, 0, n->nw[i] * 4, n->stream) ||
+            cudaMemsetAsync(l.vw, 0, n->nw[i] * 4, n->stream) ||
+            cudaMemsetAsync(l.mb, 0, s.cout * 4, n->stream) ||
+            cudaMemsetAsync(l.vb, 0, s.cout * 4, n->stream) ||
             cudaStreamSynchronize(n->stream)) {
-            delete n;
+            surr_destroy(n);
             return QLA_ECUDA;
         }
-        k_to_bf16<<<ew_blocks(n->nw[i]), 256, 0, n->stream>>>(n->wf[i], n->nw[i], n->wb[i]);
     }
-    if (cudaStreamSynchronize(n->stream) != cudaSuccess) {
-        delete n;
+    if (refresh_copies(n->prm, NCONV, n->stream) != cudaSuccess ||
+        cudaStreamSynchronize(n->stream) != cudaSuccess) {
+        surr_destroy(n);
         return QLA_ECUDA;
     }
     *out = n;
@@ -526,8 +509,8 @@ static qla_status params_io(surr_net *n, float *host, bool get, bool grads) {
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
         std::vector<float> w(n->nw[i]), b(s.cout);
-        float *dw = grads ? n->gw[i] : n->wf[i];
-        float *db = grads ? n->gb[i] : n->bias[i];
+        float *dw = grads ? n->prm.l[i].gw : n->prm.l[i].w;
+        float *db = grads ? n->prm.l[i].gb : n->prm.l[i].b;
         if (get || true) {
             NCUDA(n, cudaMemcpyAsync(w.data(), dw, n->nw[i] * 4, cudaMemcpyDeviceToHost, n->stream),
                   "surrogate: params");
@@ -552,9 +535,12 @@ static qla_status params_io(surr_net *n, float *host, bool get, bool grads) {
                   "surrogate: params");
             NCUDA(n, cudaMemcpyAsync(db, b.data(), s.cout * 4, cudaMemcpyHostToDevice, n->stream),
                   "surrogate: params");
-            k_to_bf16<<<ew_blocks(n->nw[i]), 256, 0, n->stream>>>(n->wf[i], n->nw[i], n->wb[i]);
             NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
         }
+    }
+    if (!get) {
+        NCUDA(n, refresh_copies(n->prm, NCONV, n->stream), "surrogate: params");
+        NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
     }
     return QLA_OK;
 }
@@ -569,45 +555,38 @@ qla_status surr_forward(surr_net *n, const float *feat_dev, int B, float *out_de
     qla_status s = check_batch(n, B);
     if (s != QLA_OK) return s;
     if ((s = pack(n, feat_dev, B)) != QLA_OK) return s;
-    if ((s = forward(n, B)) != QLA_OK) return s;
-    const long long P = pixels(n, B, 0);
-    k_strip<<<ew_blocks(P * NOUT), 256, 0, n->stream>>>(n->Y, CPAD, NOUT, P, out_dev);
-    NCUDA(n, cudaGetLastError(), "surrogate: strip");
-    return QLA_OK;
+    return forward(n, B, out_dev);
 }
 
 qla_status surr_loss_grad(surr_net *n, const float *feat_dev, const float *target_dev, int B,
                           double *loss_out, float *grad_host) {
     if (!n || !feat_dev || !target_dev) return QLA_EINVAL;
-    qla_status s = check_batch(n, B);
+    qla_status s = enqueue_grad(n, feat_dev, target_dev, B);
     if (s != QLA_OK) return s;
-    if ((s = pack(n, feat_dev, B)) != QLA_OK) return s;
-    if ((s = forward(n, B)) != QLA_OK) return s;
     double l = 0.0;
-    if ((s = loss(n, B, target_dev, &l)) != QLA_OK) return s;
+    if ((s = loss_end(n, &l)) != QLA_OK) return s;
     if (loss_out) *loss_out = l;
-    if ((s = backward(n, B)) != QLA_OK) return s;
     if (grad_host) return params_io(n, grad_host, true, true);
     return QLA_OK;
 }
 
+// The whole step is enqueued before the host waits for the loss, so the GPU
+// does not idle between the loss and the backward pass; Adam skips its update
+// if a convolution's wait ran out.
 qla_status surr_train_step(surr_net *n, const float *feat_dev, const float *target_dev, int B,
                            float lr, double *loss_out) {
-    qla_status s = surr_loss_grad(n, feat_dev, target_dev, B, loss_out, nullptr);
+    if (!n || !feat_dev || !target_dev) return QLA_EINVAL;
+    qla_status s = enqueue_grad(n, feat_dev, target_dev, B);
     if (s != QLA_OK) return s;
-    n->step++;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = float(1.0 - std::pow(0.9, double(n->step)));
-    const float c2 = float(1.0 - std::pow(0.999, double(n->step)));
-    for (int i = 0; i < NCONV; ++i) {
-        const ConvSpec sp = spec(i);
-        k_adam<<<ew_blocks(n->nw[i]), 256, 0, n->stream>>>(n->wf[i], n->gw[i], n->mw[i], n->vw[i],
-                                                           n->nw[i], lr, b1, b2, eps, c1, c2,
-                                                           n->wb[i]);
-        k_adam<<<1, 256, 0, n->stream>>>(n->bias[i], n->gb[i], n->mb[i], n->vb[i], sp.cout, lr, b1,
-                                         b2, eps, c1, c2, nullptr);
-    }
-    NCUDA(n, cudaGetLastError(), "surrogate: adam");
+    const double step = double(n->step + 1);
+    const float c1 = float(1.0 - std::pow(0.9, step));
+    const float c2 = float(1.0 - std::pow(0.999, step));
+    NCUDA(n, adam(n->prm, NCONV, lr, b1, b2, eps, c1, c2, n->flag, n->stream), "surrogate: adam");
+    double l = 0.0;
+    if ((s = loss_end(n, &l)) != QLA_OK) return s;
+    n->step++;
+    if (loss_out) *loss_out = l;
     return QLA_OK;
 }
 
@@ -616,6 +595,8 @@ const char *surr_last_error(const surr_net *n) { return n ? n->err.c_str() : "nu
 void surr_destroy(surr_net *n) {
     if (!n) return;
     cudaStreamSynchronize(n->stream);
+    if (n->ldone) cudaEventDestroy(n->ldone);
+    if (n->lhost) cudaFreeHost(n->lhost);
     delete n;
 }
 
@@ -681,15 +662,48 @@ qla_status surr_advance(qla_ctx *c, surr_net *n, int windows, int K, double ener
 // Direct access to the two contraction kernels, for exactness tests: with
 // BF16 inputs their only rounding is the FP32 accumulation.
 // ---------------------------------------------------------------------------
+namespace {
+// Stream-ordered scratch, given back on every path.
+struct Scratch {
+    cudaStream_t st;
+    void *p = nullptr;
+    explicit Scratch(cudaStream_t s) : st(s) {}
+    ~Scratch() { if (p) cudaFreeAsync(p, st); }
+    template <typename T> T *get(size_t n) {
+        return cudaMallocAsync(&p, n * sizeof(T), st) == cudaSuccess ? static_cast<T *>(p)
+                                                                     : nullptr;
+    }
+};
+}  // namespace
+
 extern "C" qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W, int cin,
                                        const void *w_bf16, int cout, float *out_f32,
                                        void *cuda_stream) {
     if (!in_bf16 || !w_bf16 || !out_f32 || B < 1 || H < 1 || W < 1 || cin % 32 || cout % 32)
         return QLA_EINVAL;
-    ConvArgs a{static_cast<const bf16 *>(in_bf16), B, H, W, cin, static_cast<const bf16 *>(w_bf16),
-               cout, nullptr, nullptr, nullptr, out_f32};
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (conv3x3(a, OUT_F32, false, false, st) != cudaSuccess) return QLA_ECUDA;
+    Scratch sx(st), sw(st), so(st);
+    bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));
+    bf16 *w = sw.get<bf16>(size_t(cout) * 9 * cin);
+    float *o = so.get<float>(size_t(B) * H * W * cout);
+    if (!x || !w || !o) {
+        cudaGetLastError();
+        return QLA_ECUDA;
+    }
+    ConvArgs a{};
+    a.in = x;
+    a.B = B;
+    a.H = H;
+    a.W = W;
+    a.cin = cin;
+    a.cout = cout;
+    a.w = w;
+    a.out_f = o;
+    if (nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) != cudaSuccess ||
+        block_weights(static_cast<const bf16 *>(w_bf16), cout, cin, w, st) != cudaSuccess ||
+        conv3x3(a, EP_F32, st) != cudaSuccess ||
+        blocked_to_nhwc_f32(o, B, H, W, cout, out_f32, st) != cudaSuccess)
+        return QLA_ECUDA;
     int flag = 0;
     if (cudaStreamSynchronize(st) != cudaSuccess || conv_tc_error(&flag, true) != cudaSuccess)
         return QLA_ECUDA;
@@ -706,9 +720,20 @@ extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_b
     if (!dz_bf16 || !in_bf16 || !part || !dw_f32 || cin % 32 || cout % 32 || splits < 1)
         return QLA_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (weight_grad(static_cast<const bf16 *>(dz_bf16), static_cast<const bf16 *>(in_bf16), B, H, W,
-                    cout, cin, splits, part, st) != cudaSuccess)
+    Scratch sz(st), sx(st);
+    bf16 *z = sz.get<bf16>(blocked_elems(B, cout, H, W));
+    bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));
+    if (!z || !x) {
+        cudaGetLastError();
         return QLA_ECUDA;
-    return sum_splits(part, splits, (long long)cout * 9 * cin, dw_f32, st) == cudaSuccess
+    }
+    SumJobs jobs{};
+    jobs.j[0] = {part, dw_f32, splits, (long long)cout * 9 * cin, false};
+    return nhwc_to_blocked(static_cast<const bf16 *>(dz_bf16), B, H, W, cout, z, st) ==
+                       cudaSuccess &&
+                   nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) ==
+                       cudaSuccess &&
+                   weight_grad(z, x, B, H, W, cout, cin, splits, part, st) == cudaSuccess &&
+                   sum_splits(jobs, 1, st) == cudaSuccess
                ? QLA_OK : QLA_ECUDA;
 }

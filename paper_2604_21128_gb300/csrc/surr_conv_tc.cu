@@ -52,7 +52,9 @@ constexpr int PROWS = TY + 2, PCOLS = TX + 2;       // patch rows, pixels per ro
 constexpr int PROW_BYTES = PCOLS * 16;              // 160
 constexpr int PGROUP_BYTES = PROWS * PROW_BYTES;    // 2880
 constexpr int MAX_A = 16, MAX_B = 96;               // slots of the two rings
-constexpr int CONV_THREADS = 192;                   // 4 epilogue warps, loader, MMA
+constexpr int EPI_WARPS = 8;                        // two per quarter of the TMEM lanes
+constexpr int LOAD_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1;
+constexpr int CONV_THREADS = 32 * (EPI_WARPS + 2);
 
 __device__ int g_conv_tc_error;
 // Test hook (surr_test_stall_conv): CTA 0 of each launch waits for a phase
@@ -129,40 +131,107 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 // slots of kg channel groups, na and nb ring slots (nb = every unit of a tile
 // when resident), tiles per image row / column / launch, chunk_major order.
 struct ConvPlan {
-    int nt, slices, kg, chunks, na, nb, resident, chunk_major;
+    int nt, slices, kg, chunks, na, nb, resident, chunk_major, wbox;
     int ntx, nty, tiles, tcols;
 };
 
-// The accumulator row of this thread (TMEM lane, pixel (y, x) of image b),
-// output channels co0 .. co0 + nt - 1, by mode.  Every thread of the warp takes
-// part in the loads and shuffles; only pixels of the image store.
-template <ConvMode MODE>
-__device__ __forceinline__ void epilogue(const ConvArgs &a, uint32_t tmem_row, int nt, int co0,
-                                         int b, int y, int x) {
+// Store to a blocked plane's pixel r with the halo copies that `edge` names:
+// bits 0-3: first column, last column, first row, last row of the image.
+__device__ __forceinline__ void put_edge(uint4 *r, unsigned edge, int H, int W, uint4 v) {
+    *r = v;
+    if (edge == 0) return;
+    const long long col = (long long)H * (W + 2);
+    if (edge & 1) r[W] = v;
+    if (edge & 2) r[-W] = v;
+    if (edge & 4) {
+        uint4 *q = r + col;
+        *q = v;
+        if (edge & 1) q[W] = v;
+        if (edge & 2) q[-W] = v;
+    }
+    if (edge & 8) {
+        uint4 *q = r - col;
+        *q = v;
+        if (edge & 1) q[W] = v;
+        if (edge & 2) q[-W] = v;
+    }
+}
+__device__ __forceinline__ unsigned edge_of(int y, int x, int H, int W) {
+    return (x == 0 ? 1u : 0u) | (x == W - 1 ? 2u : 0u) | (y == 0 ? 4u : 0u) |
+           (y == H - 1 ? 8u : 0u);
+}
+
+// Output channels [c_lo, c_hi) of co0's tile for this thread's accumulator
+// row (TMEM lane, pixel (y, x) of image b), by mode; `wait` returns once the
+// accumulator is complete (false: give up).  bias points to the tile's biases
+// in shared memory.  Every thread of the warp takes part in the loads and
+// shuffles; only pixels of the image store.  What does not depend on the
+// accumulator (addresses, edges, the first skip values) comes before the wait.
+template <ConvMode MODE, typename Wait>
+__device__ __forceinline__ bool epilogue(const ConvArgs &a, uint32_t tmem_row, int c_lo, int c_hi,
+                                         int co0, const float *bias, int b, int y, int x,
+                                         Wait wait) {
     const bool valid = y < a.H && x < a.W;
-    const int G = a.cout / 8;
+    const int G = a.cout / 8, g0 = (co0 + c_lo) / 8;
+    if constexpr (MODE == EP_F32) {
+        float4 *o = reinterpret_cast<float4 *>(a.out_f) +
+                    2 * (((size_t(b) * G + g0) * a.H + y) * a.W + x);
+        const size_t step = 2 * size_t(a.H) * a.W;
+        if (!wait()) return false;
 #pragma unroll 1
-    for (int c0 = 0; c0 < nt; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem_row + uint32_t(c0), v);
-        const int co = co0 + c0;
-        if constexpr (MODE == EP_F32) {
-            if (!valid) continue;
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+            float v[16];
+            tmem_ld16(tmem_row + uint32_t(c0), v);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const size_t u = ((size_t(b) * G + co / 8 + h) * a.H + y) * a.W + x;
-                float4 *o = reinterpret_cast<float4 *>(a.out_f) + 2 * u;
+            for (int h = 0; h < 2; ++h, o += step) {
+                if (!valid) continue;
                 o[0] = make_float4(v[8 * h], v[8 * h + 1], v[8 * h + 2], v[8 * h + 3]);
                 o[1] = make_float4(v[8 * h + 4], v[8 * h + 5], v[8 * h + 6], v[8 * h + 7]);
             }
-        } else if constexpr (MODE == EP_OUT) {
+        }
+    } else if constexpr (MODE == EP_OUT) {
+        float *o = a.out_f + ((size_t(b) * a.H + y) * a.W + x) * a.n_out;
+        if (!wait()) return false;
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+            float v[16];
+            tmem_ld16(tmem_row + uint32_t(c0), v);
             if (!valid) continue;
-            float *o = a.out_f + ((size_t(b) * a.H + y) * a.W + x) * a.n_out;
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-                if (co + j < a.n_out) o[co + j] = v[j] + a.bias[co + j];
-        } else {
-            const float4 *bb = reinterpret_cast<const float4 *>(a.bias + co);
+                if (co0 + c0 + j < a.n_out) o[co0 + c0 + j] = v[j] + bias[c0 + j];
+        }
+    } else {
+        const size_t step = plane8(0, 1, 1, a.H, a.W);
+        const size_t at = plane8(b, g0, G, a.H, a.W) + pixel8(y, x, a.W);
+        const uint4 *sk = reinterpret_cast<const uint4 *>(a.skip) + at;
+        uint4 *o = reinterpret_cast<uint4 *>(a.out) + at;
+        const unsigned edge = edge_of(y, x, a.H, a.W);
+        const int h2 = a.H / 2, w2 = a.W / 2, H2 = 2 * a.H, W2 = 2 * a.W;
+        const size_t pstep = plane8(0, 1, 1, h2, w2), ustep = plane8(0, 1, 1, H2, W2);
+        uint4 *po = reinterpret_cast<uint4 *>(a.pool) + plane8(b, g0, G, h2, w2) +
+                    pixel8(y / 2, x / 2, w2);
+        const unsigned pedge = edge_of(y / 2, x / 2, h2, w2);
+        uint4 *uo = reinterpret_cast<uint4 *>(a.up) + plane8(b, g0, G, H2, W2) +
+                    pixel8(2 * y, 2 * x, W2);
+        const bool skip = a.skip && valid;
+        uint4 s0 = make_uint4(0, 0, 0, 0), s1 = s0;
+        if (skip) {
+            s0 = sk[0];
+            s1 = sk[step];
+        }
+        if (!wait()) return false;
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+            float v[16];
+            tmem_ld16(tmem_row + uint32_t(c0), v);
+            const uint4 sv[2] = {s0, s1};
+            if (skip && c0 + 16 < c_hi) {   // the next channels' skip values
+                sk += 2 * step;
+                s0 = sk[0];
+                s1 = sk[step];
+            }
+            const float4 *bb = reinterpret_cast<const float4 *>(bias + c0);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float4 t = bb[j];
@@ -173,33 +242,34 @@ __device__ __forceinline__ void epilogue(const ConvArgs &a, uint32_t tmem_row, i
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int g = co / 8 + h;
-                float o[8];
+                float q[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) o[j] = v[8 * h + j];
-                if (a.skip && valid) {
+                for (int j = 0; j < 8; ++j) q[j] = v[8 * h + j];
+                if (a.skip) {
                     float s[8];
-                    unpack8(reinterpret_cast<const uint4 *>(a.skip)[plane8(b, g, G, a.H, a.W) +
-                                                                    pixel8(y, x, a.W)], s);
+                    unpack8(sv[h], s);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) o[j] += s[j];
+                    for (int j = 0; j < 8; ++j) q[j] += s[j];
                 }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) o[j] = o[j] > 0.f ? o[j] : LEAK * o[j];
-                const uint4 r = pack8(o);
-                if (valid)
-                    put8(reinterpret_cast<uint4 *>(a.out) + plane8(b, g, G, a.H, a.W), y, x, a.H,
-                         a.W, r);
-                if (a.up && valid) {
-                    uint4 *p = reinterpret_cast<uint4 *>(a.up) + plane8(b, g, G, 2 * a.H, 2 * a.W);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        put8(p, 2 * y + (k >> 1), 2 * x + (k & 1), 2 * a.H, 2 * a.W, r);
+                for (int j = 0; j < 8; ++j) q[j] = q[j] > 0.f ? q[j] : LEAK * q[j];
+                const uint4 r = pack8(q);
+                if (valid) put_edge(o, edge, a.H, a.W, r);
+                o += step;
+                if (a.up) {
+                    if (valid) {
+                        // the four copies touch the halo where this pixel does
+                        put_edge(uo, edge & 5, H2, W2, r);
+                        put_edge(uo + 1, edge & 6, H2, W2, r);
+                        put_edge(uo + W2 + 2, edge & 9, H2, W2, r);
+                        put_edge(uo + W2 + 3, edge & 10, H2, W2, r);
+                    }
+                    uo += ustep;
                 }
                 if (a.pool) {
                     // the tile's rows are eight lanes apart, its columns one;
                     // tiles start on even pixels
-                    const auto at = [&](int d) {
+                    const auto lane_at = [&](int d) {
                         return make_uint4(__shfl_down_sync(0xffffffffu, r.x, d),
                                           __shfl_down_sync(0xffffffffu, r.y, d),
                                           __shfl_down_sync(0xffffffffu, r.z, d),
@@ -207,29 +277,30 @@ __device__ __forceinline__ void epilogue(const ConvArgs &a, uint32_t tmem_row, i
                     };
                     float p0[8], p1[8], p2[8], p3[8];
                     unpack8(r, p0);
-                    unpack8(at(1), p1);
-                    unpack8(at(8), p2);
-                    unpack8(at(9), p3);
+                    unpack8(lane_at(1), p1);
+                    unpack8(lane_at(8), p2);
+                    unpack8(lane_at(9), p3);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) o[j] = 0.25f * (p0[j] + p1[j] + p2[j] + p3[j]);
-                    if (valid && !(y & 1) && !(x & 1))
-                        put8(reinterpret_cast<uint4 *>(a.pool) +
-                                 plane8(b, g, G, a.H / 2, a.W / 2),
-                             y / 2, x / 2, a.H / 2, a.W / 2, pack8(o));
+                    for (int j = 0; j < 8; ++j) q[j] = 0.25f * (p0[j] + p1[j] + p2[j] + p3[j]);
+                    if (valid && !(y & 1) && !(x & 1)) put_edge(po, pedge, h2, w2, pack8(q));
+                    po += pstep;
                 }
             }
         }
     }
+    return true;
 }
 
 template <ConvMode MODE>
 __global__ void __launch_bounds__(CONV_THREADS)
-k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const ConvPlan pl) {
+k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap wmap,
+          const ConvArgs a, const ConvPlan pl) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_a[MAX_A], empty_a[MAX_A], full_b[MAX_B], empty_b[MAX_B];
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ __align__(16) float bias_s[256];
 
     // the warp index through a shuffle: its branches are then uniform
     const int tid = threadIdx.x, lane = tid & 31;
@@ -255,12 +326,14 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
         }
         for (int k = 0; k < 2; ++k) {
             mbar_init(&acc_full[k], 1);
-            mbar_init(&acc_empty[k], 4);
+            mbar_init(&acc_empty[k], EPI_WARPS);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
     }
-    if (warp == 5) {
+    if constexpr (MODE != EP_F32)
+        if (tid < pl.nt) bias_s[tid] = a.bias[co0 + tid];
+    if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_slot)),
                      "r"(pl.tcols)
@@ -272,7 +345,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 4 && lane == 0) {
+    if (warp == LOAD_WARP && lane == 0) {
         // loader: patches and weight units in the order the MMAs take them
         // (ring positions step; divisions would cost as much as a unit's MMAs)
         int as = 0, bs = 0, na_used = 0, nb_used = 0;   // slots, and how many ever filled
@@ -296,7 +369,10 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
             mbar_expect_tx(&full_b[bs], uint32_t(b_bytes));
             const bf16 *src = a.w + tap * w_tap + c * pl.kg * w_group + co0 * 8;
             unsigned char *dst = sb + bs * b_bytes;
+            // one copy per unit: contiguous if it has every output channel,
+            // else a box of channels x channel groups
             if (pl.slices == 1) bulk_load(dst, src, uint32_t(b_bytes), &full_b[bs]);
+            else if (pl.wbox) tma_load_2d(dst, &wmap, co0 * 2, tap * (a.cin / 8) + c * pl.kg, &full_b[bs]);
             else
                 for (int g = 0; g < pl.kg; ++g)
                     bulk_load(dst + g * w_bytes, src + g * w_group, w_bytes, &full_b[bs]);
@@ -333,7 +409,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
             if (bs == 0) { bs = pl.nb; bp ^= 1; }
             mbar_wait(&full_b[--bs], bp ^ 1);
         }
-    } else if (warp == 5) {
+    } else if (warp == MMA_WARP) {
         // The whole warp runs the loop, one elected lane issues: branches and
         // descriptors are then uniform.  Descriptors step by precomputed
         // offsets: a unit's two MMAs take 80 (N = 32) to 256 cycles, which a
@@ -376,7 +452,26 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
                 if (++bs == pl.nb) { bs = 0; bp ^= 1; }
             };
             constexpr uint32_t ROW = PROW_BYTES / 16;
-            if (pl.chunk_major) {
+            if (pl.chunk_major && !weights) {
+                // resident weights: nothing to wait for within a patch
+                for (int c = 0; c < pl.chunks; ++c) {
+                    wait(&full_a[as], ap);
+                    if (!ok) break;
+                    if (leader) {
+                        const uint64_t da = a0 + uint64_t(as * a_step);
+                        uint64_t db = b0 + uint64_t(c * 9 * b_step);
+#pragma unroll
+                        for (int tap = 0; tap < 9; ++tap, db += b_step) {
+                            const uint32_t off = (tap / 3) * ROW + tap % 3;
+                            umma(d, da + off, db, idesc, tap > 0 ? 1 : acc);
+                            if (two) umma(d, da + (off + 2 * PGROUP_BYTES / 16), db + bk, idesc, 1);
+                        }
+                        umma_commit(&empty_a[as]);
+                    }
+                    acc = 1;
+                    if (++as == pl.na) { as = 0; ap ^= 1; }
+                }
+            } else if (pl.chunk_major) {
                 for (int c = 0; c < pl.chunks && ok; ++c) {
                     wait(&full_a[as], ap);
                     if (!ok) break;
@@ -405,21 +500,28 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
             if (ok && leader) umma_commit(&acc_full[buf]);
         }
         if (!ok) abort_flag = 1;
-    } else if (warp < 4) {
+    } else if (warp < EPI_WARPS) {
+        // warps w and w + 4 share TMEM lanes and split the channels
+        const int part = warp >> 2, row = (warp & 3) * 32 + lane;
+        const int c_lo = pl.nt >= 32 ? part * (pl.nt / 2) : 0;
+        const int c_hi = pl.nt >= 32 ? c_lo + pl.nt / 2 : part == 0 ? pl.nt : 0;
         bool ok = true;
         for (int k = 0; k < items && ok; ++k) {
             const int buf = k & 1;
-            ok = mbar_wait(&acc_full[buf], (k / 2) & 1, abort);
-            // tcgen05.ld is warp-collective: decide for the whole warp
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
             int t = first + k * stride;
             const int tx = t % pl.ntx;
             t /= pl.ntx;
             const int ty = t % pl.nty, b = t / pl.nty;
-            epilogue<MODE>(a, tmem + uint32_t(buf * pl.nt) + (uint32_t(warp * 32) << 16), pl.nt,
-                           co0, b, ty * TY + (tid >> 3), tx * TX + (tid & 7));
+            ok = epilogue<MODE>(
+                a, tmem + uint32_t(buf * pl.nt) + (uint32_t((warp & 3) * 32) << 16), c_lo, c_hi,
+                co0, bias_s, b, ty * TY + (row >> 3), tx * TX + (row & 7), [&] {
+                    // tcgen05.ld is warp-collective: decide for the whole warp
+                    const bool f = __all_sync(0xffffffffu,
+                                              mbar_wait(&acc_full[buf], (k / 2) & 1, abort));
+                    tc_fence_after();
+                    return f;
+                });
+            if (!ok) break;
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
@@ -433,7 +535,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const ConvArgs a, const Conv
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && abort_flag) atomicExch(&g_conv_tc_error, 1);
-    if (warp == 5)
+    if (warp == MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(pl.tcols)
                      : "memory");
@@ -456,6 +558,21 @@ EncodeTiled encode_tiled() {
         return reinterpret_cast<EncodeTiled>(p);
     }();
     return fn;
+}
+
+// Weights [tap][cin / 8][cout][8] as rows of output channels: boxes of nt
+// channels x kg groups.
+bool weight_map(CUtensorMap *map, const bf16 *w, int cout, int cin, int nt, int kg) {
+    const EncodeTiled enc = encode_tiled();
+    if (!enc || (reinterpret_cast<uintptr_t>(w) & 15)) return false;
+    const cuuint64_t dims[2] = {cuuint64_t(cout) * 2, cuuint64_t(9 * (cin / 8))};
+    const cuuint64_t strides[1] = {cuuint64_t(cout) * 16};
+    const cuuint32_t box[2] = {cuuint32_t(nt * 2), cuuint32_t(kg)};
+    const cuuint32_t estr[2] = {1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<bf16 *>(w), dims, strides, box,
+               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Streaming multiprocessors of the current device, read once.
@@ -502,7 +619,7 @@ bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
     pl->chunk_major = a.W % 128 == 0 || pl->chunks + 1 > MAX_A;
     const int need = pl->chunk_major ? 1 : pl->chunks;
     // two CTAs per SM where weights and a few patches fit twice, else one;
-    // weights resident where they fit, else a ring of about 64 KB
+    // weights resident where they fit, else a ring of what is left
     for (int c = 2; c >= 1; --c) {
         const int budget = (c == 2 ? 110 : 222) * 1024;
         if (pl->tcols * c > 512) continue;
@@ -512,11 +629,12 @@ bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
             pl->na = std::min(std::min(MAX_A, std::max(4, 2 * need)),
                               (budget - units * b_bytes) / a_bytes);
         } else if (c == 1) {
+            // two patches ahead, weights in the rest: at 8 KB a unit, eight
+            // slots covered a third of the L2 latency of a unit's load
             pl->resident = 0;
-            pl->nb = std::max(3, std::min(std::min(units, 16), 65536 / b_bytes));
-            pl->na = std::min(MAX_A, (budget - pl->nb * b_bytes) / a_bytes);
-            if (pl->na < need) return false;
-            pl->na = std::min(pl->na, std::max(4, 2 * need));
+            pl->na = std::min(MAX_A, need + 2);
+            pl->nb = std::min(std::min(units, MAX_B), (budget - pl->na * a_bytes) / b_bytes);
+            if (pl->nb < 3) return false;
         } else {
             continue;
         }
@@ -545,10 +663,14 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st) {
     if (!plan_conv(a, &pl, &smem, &per_sm)) return cudaErrorInvalidConfiguration;
     if (!blocked_map(&map, a.in, a.B, a.cin, a.H, a.W, true, PCOLS, PROWS, pl.kg))
         return cudaErrorNotSupported;
+    pl.wbox = pl.slices > 1 && pl.nt <= 128;
+    CUtensorMap wmap = map;
+    if (pl.wbox && !weight_map(&wmap, a.w, a.cout, a.cin, pl.nt, pl.kg))
+        return cudaErrorNotSupported;
     // whole slices: every slice gets the same number of CTAs
     int per_slice = std::max(1, sm_count() * per_sm / pl.slices);
     if (per_slice > pl.tiles) per_slice = pl.tiles;
-    k<<<unsigned(per_slice) * unsigned(pl.slices), CONV_THREADS, smem, st>>>(map, a, pl);
+    k<<<unsigned(per_slice) * unsigned(pl.slices), CONV_THREADS, smem, st>>>(map, wmap, a, pl);
     return cudaGetLastError();
 }
 

@@ -112,6 +112,9 @@ __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
 // mbarriers and TMA.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // a wait gives up after 2 s
+// How long one try may suspend the thread: waiting warps that poll instead
+// slow down the warps they wait for.
+constexpr unsigned TRY_NS = 1000000;
 
 __device__ __forceinline__ void mbar_init(uint64_t *b, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count)
@@ -129,10 +132,10 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
-        : "r"(a), "r"(parity)
+        : "r"(a), "r"(parity), "r"(TRY_NS)
         : "memory");
     return done != 0;
 }

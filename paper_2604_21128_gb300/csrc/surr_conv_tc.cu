@@ -128,33 +128,41 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 }
 
 // How a launch is laid out: NT output channels per tile (cout / NT slices),
-// slots of kg channel groups, na and nb ring slots (nb = every unit of a tile
-// when resident), tiles per image row / column / launch, chunk_major order.
+// patches of kg channel groups, weight units of one tap and bc patches, na
+// and nb ring slots (nb = every unit of a tile when resident), tiles per image
+// row / column / launch, chunk_major order.
 struct ConvPlan {
-    int nt, slices, kg, chunks, na, nb, resident, chunk_major, wbox;
+    int nt, slices, kg, chunks, bc, na, nb, resident, chunk_major, wbox;
     int ntx, nty, tiles, tcols;
 };
 
-// Store to a blocked plane's pixel r with the halo copies that `edge` names:
-// bits 0-3: first column, last column, first row, last row of the image.
-__device__ __forceinline__ void put_edge(uint4 *r, unsigned edge, int H, int W, uint4 v) {
+// Store at *r, part of a pixel of a blocked plane (u parts per pixel), with
+// the halo copies that `edge` names: bits 0-3: first column, last column,
+// first row, last row of the image.
+template <typename V>
+__device__ __forceinline__ void put_edge(V *r, int u, unsigned edge, int H, int W, V v) {
     *r = v;
     if (edge == 0) return;
-    const long long col = (long long)H * (W + 2);
-    if (edge & 1) r[W] = v;
-    if (edge & 2) r[-W] = v;
+    const long long col = (long long)H * (W + 2) * u, row = (long long)W * u;
+    if (edge & 1) r[row] = v;
+    if (edge & 2) r[-row] = v;
     if (edge & 4) {
-        uint4 *q = r + col;
+        V *q = r + col;
         *q = v;
-        if (edge & 1) q[W] = v;
-        if (edge & 2) q[-W] = v;
+        if (edge & 1) q[row] = v;
+        if (edge & 2) q[-row] = v;
     }
     if (edge & 8) {
-        uint4 *q = r - col;
+        V *q = r - col;
         *q = v;
-        if (edge & 1) q[W] = v;
-        if (edge & 2) q[-W] = v;
+        if (edge & 1) q[row] = v;
+        if (edge & 2) q[-row] = v;
     }
+}
+__device__ __forceinline__ float2 unpack2(uint32_t w) {
+    __nv_bfloat162 b;
+    *reinterpret_cast<uint32_t *>(&b) = w;
+    return make_float2(__bfloat162float(b.x), __bfloat162float(b.y));
 }
 __device__ __forceinline__ unsigned edge_of(int y, int x, int H, int W) {
     return (x == 0 ? 1u : 0u) | (x == W - 1 ? 2u : 0u) | (y == 0 ? 4u : 0u) |
@@ -215,10 +223,14 @@ __device__ __forceinline__ bool epilogue(const ConvArgs &a, uint32_t tmem_row, i
         uint4 *uo = reinterpret_cast<uint4 *>(a.up) + plane8(b, g0, G, H2, W2) +
                     pixel8(2 * y, 2 * x, W2);
         const bool skip = a.skip && valid;
-        uint4 s0 = make_uint4(0, 0, 0, 0), s1 = s0;
+        uint4 s0 = make_uint4(0, 0, 0, 0), s1 = s0, s2 = s0, s3 = s0;
         if (skip) {
             s0 = sk[0];
             s1 = sk[step];
+            if (c_lo + 16 < c_hi) {
+                s2 = sk[2 * step];
+                s3 = sk[3 * step];
+            }
         }
         if (!wait()) return false;
 #pragma unroll 1
@@ -226,10 +238,12 @@ __device__ __forceinline__ bool epilogue(const ConvArgs &a, uint32_t tmem_row, i
             float v[16];
             tmem_ld16(tmem_row + uint32_t(c0), v);
             const uint4 sv[2] = {s0, s1};
-            if (skip && c0 + 16 < c_hi) {   // the next channels' skip values
+            s0 = s2;
+            s1 = s3;
+            if (skip && c0 + 32 < c_hi) {   // skip values two rounds ahead
+                s2 = sk[4 * step];
+                s3 = sk[5 * step];
                 sk += 2 * step;
-                s0 = sk[0];
-                s1 = sk[step];
             }
             const float4 *bb = reinterpret_cast<const float4 *>(bias + c0);
 #pragma unroll
@@ -254,35 +268,41 @@ __device__ __forceinline__ bool epilogue(const ConvArgs &a, uint32_t tmem_row, i
 #pragma unroll
                 for (int j = 0; j < 8; ++j) q[j] = q[j] > 0.f ? q[j] : LEAK * q[j];
                 const uint4 r = pack8(q);
-                if (valid) put_edge(o, edge, a.H, a.W, r);
+                if (valid) put_edge(o, 1, edge, a.H, a.W, r);
                 o += step;
                 if (a.up) {
                     if (valid) {
                         // the four copies touch the halo where this pixel does
-                        put_edge(uo, edge & 5, H2, W2, r);
-                        put_edge(uo + 1, edge & 6, H2, W2, r);
-                        put_edge(uo + W2 + 2, edge & 9, H2, W2, r);
-                        put_edge(uo + W2 + 3, edge & 10, H2, W2, r);
+                        put_edge(uo, 1, edge & 5, H2, W2, r);
+                        put_edge(uo + 1, 1, edge & 6, H2, W2, r);
+                        put_edge(uo + W2 + 2, 1, edge & 9, H2, W2, r);
+                        put_edge(uo + W2 + 3, 1, edge & 10, H2, W2, r);
                     }
                     uo += ustep;
                 }
                 if (a.pool) {
-                    // the tile's rows are eight lanes apart, its columns one;
-                    // tiles start on even pixels
-                    const auto lane_at = [&](int d) {
-                        return make_uint4(__shfl_down_sync(0xffffffffu, r.x, d),
-                                          __shfl_down_sync(0xffffffffu, r.y, d),
-                                          __shfl_down_sync(0xffffffffu, r.z, d),
-                                          __shfl_down_sync(0xffffffffu, r.w, d));
-                    };
-                    float p0[8], p1[8], p2[8], p3[8];
-                    unpack8(r, p0);
-                    unpack8(lane_at(1), p1);
-                    unpack8(lane_at(8), p2);
-                    unpack8(lane_at(9), p3);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) q[j] = 0.25f * (p0[j] + p1[j] + p2[j] + p3[j]);
-                    if (valid && !(y & 1) && !(x & 1)) put_edge(po, pedge, h2, w2, pack8(q));
+                    // The tile's columns are one lane apart, its rows eight,
+                    // and tiles start on even pixels: the four lanes of a
+                    // pooled pixel swap words until each holds two channels
+                    // of all four pixels.
+                    const bool xo = x & 1, yo = y & 1;
+                    const uint32_t k0 = xo ? r.z : r.x, k1 = xo ? r.w : r.y;
+                    const uint32_t m0 = __shfl_xor_sync(0xffffffffu, xo ? r.x : r.z, 1);
+                    const uint32_t m1 = __shfl_xor_sync(0xffffffffu, xo ? r.y : r.w, 1);
+                    // (l, r): the row's left and right pixel, words 0 and 1
+                    const uint32_t l0 = xo ? m0 : k0, l1 = xo ? m1 : k1;
+                    const uint32_t r0 = xo ? k0 : m0, r1 = xo ? k1 : m1;
+                    const uint32_t nl = __shfl_xor_sync(0xffffffffu, yo ? l0 : l1, 8);
+                    const uint32_t nr = __shfl_xor_sync(0xffffffffu, yo ? r0 : r1, 8);
+                    const uint32_t ml = yo ? l1 : l0, mr = yo ? r1 : r0;
+                    const float2 p0 = unpack2(yo ? nl : ml), p1 = unpack2(yo ? nr : mr);
+                    const float2 p2 = unpack2(yo ? ml : nl), p3 = unpack2(yo ? mr : nr);
+                    const __nv_bfloat162 m =
+                        __floats2bfloat162_rn(0.25f * (p0.x + p1.x + p2.x + p3.x),
+                                              0.25f * (p0.y + p1.y + p2.y + p3.y));
+                    if (valid)
+                        put_edge(reinterpret_cast<uint32_t *>(po) + (xo ? 2 : 0) + (yo ? 1 : 0), 4,
+                                 pedge, h2, w2, *reinterpret_cast<const uint32_t *>(&m));
                     po += pstep;
                 }
             }
@@ -309,28 +329,28 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
     const int stride = int(gridDim.x) / pl.slices;
     const int co0 = slice * pl.nt;
     const int items = first < pl.tiles ? (pl.tiles - 1 - first) / stride + 1 : 0;
-    const int a_bytes = pl.kg * PGROUP_BYTES, b_bytes = pl.kg * pl.nt * 16;
+    const int a_bytes = pl.kg * PGROUP_BYTES, b_bytes = pl.bc * pl.kg * pl.nt * 16;
     // TMA destinations must be 128-byte aligned (the launch adds the slack)
     unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     unsigned char *sa = smem, *sb = smem + pl.na * a_bytes;
     const volatile int *abort = &abort_flag;
 
-    if (tid == 0) {
-        for (int k = 0; k < pl.na; ++k) {
+    if (warp == LOAD_WARP) {
+        for (int k = lane; k < pl.na; k += 32) {
             mbar_init(&full_a[k], 1);
             mbar_init(&empty_a[k], 1);
         }
-        for (int k = 0; k < pl.nb; ++k) {
+        for (int k = lane; k < pl.nb; k += 32) {
             mbar_init(&full_b[k], 1);
             mbar_init(&empty_b[k], 1);
         }
-        for (int k = 0; k < 2; ++k) {
-            mbar_init(&acc_full[k], 1);
-            mbar_init(&acc_empty[k], EPI_WARPS);
+        if (lane < 2) {
+            mbar_init(&acc_full[lane], 1);
+            mbar_init(&acc_empty[lane], EPI_WARPS);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        abort_flag = 0;
     }
+    if (tid == 0) abort_flag = 0;
     if constexpr (MODE != EP_F32)
         if (tid < pl.nt) bias_s[tid] = a.bias[co0 + tid];
     if (warp == MMA_WARP) {
@@ -374,7 +394,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
             if (pl.slices == 1) bulk_load(dst, src, uint32_t(b_bytes), &full_b[bs]);
             else if (pl.wbox) tma_load_2d(dst, &wmap, co0 * 2, tap * (a.cin / 8) + c * pl.kg, &full_b[bs]);
             else
-                for (int g = 0; g < pl.kg; ++g)
+                for (int g = 0; g < pl.bc * pl.kg; ++g)
                     bulk_load(dst + g * w_bytes, src + g * w_group, w_bytes, &full_b[bs]);
             if (++bs == pl.nb) { bs = 0; bp ^= 1; }
         };
@@ -393,7 +413,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
                 for (int tap = 0; tap < 9 && ok; ++tap)
                     for (int c = 0; c < pl.chunks && ok; ++c) {
                         if (tap == 0) load_a(c, tx, ty, b);
-                        if (weights && ok) load_b(tap, c);
+                        if (weights && ok && c % pl.bc == 0) load_b(tap, c);
                     }
             }
         }
@@ -437,65 +457,74 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
             const bool weights = stream || k == 0;   // weight units to wait for
             uint32_t acc = 0;
             if (!stream) bs = 0;
-            // unit: the MMAs of tap offset `off` on A slot sl
-            auto unit = [&](uint32_t off, int sl) {
-                if (weights) wait(&full_b[bs], stream ? bp : 0);
-                if (!ok) return;
-                const uint64_t da = a0 + uint64_t(sl * a_step + off);
-                const uint64_t db = b0 + uint64_t(bs * b_step);
-                if (leader) {
-                    umma(d, da, db, idesc, acc);
-                    if (two) umma(d, da + 2 * PGROUP_BYTES / 16, db + bk, idesc, 1);
-                    if (stream) umma_commit(&empty_b[bs]);
-                }
-                acc = 1;
-                if (++bs == pl.nb) { bs = 0; bp ^= 1; }
-            };
             constexpr uint32_t ROW = PROW_BYTES / 16;
-            if (pl.chunk_major && !weights) {
-                // resident weights: nothing to wait for within a patch
-                for (int c = 0; c < pl.chunks; ++c) {
-                    wait(&full_a[as], ap);
-                    if (!ok) break;
-                    if (leader) {
-                        const uint64_t da = a0 + uint64_t(as * a_step);
-                        uint64_t db = b0 + uint64_t(c * 9 * b_step);
-#pragma unroll
-                        for (int tap = 0; tap < 9; ++tap, db += b_step) {
-                            const uint32_t off = (tap / 3) * ROW + tap % 3;
-                            umma(d, da + off, db, idesc, tap > 0 ? 1 : acc);
-                            if (two) umma(d, da + (off + 2 * PGROUP_BYTES / 16), db + bk, idesc, 1);
-                        }
-                        umma_commit(&empty_a[as]);
-                    }
-                    acc = 1;
-                    if (++as == pl.na) { as = 0; ap ^= 1; }
-                }
-            } else if (pl.chunk_major) {
+            if (pl.chunk_major) {
                 for (int c = 0; c < pl.chunks && ok; ++c) {
                     wait(&full_a[as], ap);
                     if (!ok) break;
+                    const uint64_t da = a0 + uint64_t(as * a_step);
+                    if (!weights) {
+                        // resident weights: nothing to wait for within a patch
+                        if (leader) {
+                            uint64_t db = b0 + uint64_t(c * 9 * b_step);
 #pragma unroll
-                    for (int tap = 0; tap < 9; ++tap)
-                        if (ok) unit((tap / 3) * ROW + tap % 3, as);
+                            for (int tap = 0; tap < 9; ++tap, db += b_step) {
+                                const uint32_t off = (tap / 3) * ROW + tap % 3;
+                                umma(d, da + off, db, idesc, tap > 0 ? 1 : acc);
+                                if (two)
+                                    umma(d, da + (off + 2 * PGROUP_BYTES / 16), db + bk, idesc, 1);
+                            }
+                        }
+                        acc = 1;
+                    } else {
+#pragma unroll
+                        for (int tap = 0; tap < 9; ++tap) {
+                            const uint32_t off = (tap / 3) * ROW + tap % 3;
+                            if (ok) wait(&full_b[bs], stream ? bp : 0);
+                            if (ok && leader) {
+                                const uint64_t db = b0 + uint64_t(bs * b_step);
+                                umma(d, da + off, db, idesc, acc);
+                                if (two)
+                                    umma(d, da + (off + 2 * PGROUP_BYTES / 16), db + bk, idesc, 1);
+                                if (stream) umma_commit(&empty_b[bs]);
+                            }
+                            acc = 1;
+                            if (++bs == pl.nb) { bs = 0; bp ^= 1; }
+                        }
+                    }
                     if (ok && leader) umma_commit(&empty_a[as]);
                     if (++as == pl.na) { as = 0; ap ^= 1; }
                 }
             } else {
+                // the tile's patches are slots as .. as + chunks - 1 (na is a
+                // multiple of chunks)
 #pragma unroll 1
                 for (int tap = 0; tap < 9 && ok; ++tap) {
-                    const uint32_t off = (tap / 3) * ROW + tap % 3;
-                    int sl = as;
-                    uint32_t p = ap;
-                    for (int c = 0; c < pl.chunks && ok; ++c) {
-                        if (tap == 0) wait(&full_a[sl], p);
+                    uint64_t da = a0 + uint64_t(as * a_step + (tap / 3) * ROW + tap % 3);
+                    for (int c = 0; c < pl.chunks; c += pl.bc) {
+                        if (tap == 0)
+                            for (int e = 0; e < pl.bc && ok; ++e) wait(&full_a[as + c + e], ap);
+                        if (ok && weights) wait(&full_b[bs], stream ? bp : 0);
                         if (!ok) break;
-                        unit(off, sl);
-                        if (tap == 8 && ok && leader) umma_commit(&empty_a[sl]);
-                        if (++sl == pl.na) { sl = 0; p ^= 1; }
+                        if (leader) {
+                            uint64_t db = b0 + uint64_t(bs * b_step);
+                            // bc is 1, 2 or 4 patches
+                            for (int e = 0; e < pl.bc; ++e) {
+                                umma(d, da, db, idesc, acc);
+                                if (two) umma(d, da + 2 * PGROUP_BYTES / 16, db + bk, idesc, 1);
+                                acc = 1;
+                                da += a_step;
+                                db += 2 * bk;
+                            }
+                            if (stream) umma_commit(&empty_b[bs]);
+                        }
+                        if (++bs == pl.nb) { bs = 0; bp ^= 1; }
                     }
-                    if (tap == 8) { as = sl; ap = p; }
                 }
+                if (ok && leader)
+                    for (int c = 0; c < pl.chunks; ++c) umma_commit(&empty_a[as + c]);
+                as += pl.chunks;
+                if (as == pl.na) { as = 0; ap ^= 1; }
             }
             if (ok && leader) umma_commit(&acc_full[buf]);
         }
@@ -612,32 +641,43 @@ bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
     if (!pl->nt) return false;
     pl->slices = a.cout / pl->nt;
     pl->tcols = std::max(32, 2 * pl->nt);
-    const int units = 9 * pl->chunks;
-    const int a_bytes = pl->kg * PGROUP_BYTES, b_bytes = pl->kg * pl->nt * 16;
     // slots of a tile that must be resident together: all of them when the
-    // taps are outermost
-    pl->chunk_major = a.W % 128 == 0 || pl->chunks + 1 > MAX_A;
+    // taps are outermost; a weight unit then covers four patches (eight MMAs
+    // per wait: with two, the waits and ring steps of a single warp, 400 to
+    // 500 cycles per unit, took longer than the MMAs)
+    pl->chunk_major = a.W % 128 == 0 || pl->chunks > MAX_A;
     const int need = pl->chunk_major ? 1 : pl->chunks;
+    pl->bc = 1;
+    const int a_bytes = pl->kg * PGROUP_BYTES;
+    // (four ring slots of it have to fit beside a tile's patches)
+    if (!pl->chunk_major)
+        while (pl->bc < 4 && pl->chunks % (2 * pl->bc) == 0 &&
+               4 * (2 * pl->bc * pl->kg * pl->nt * 16) + need * a_bytes <= 222 * 1024)
+            pl->bc *= 2;
+    const int units = 9 * pl->chunks / pl->bc;
+    const int b_bytes = pl->bc * pl->kg * pl->nt * 16;
     // two CTAs per SM where weights and a few patches fit twice, else one;
     // weights resident where they fit, else a ring of what is left
     for (int c = 2; c >= 1; --c) {
         const int budget = (c == 2 ? 110 : 222) * 1024;
         if (pl->tcols * c > 512) continue;
-        if (units <= MAX_B && units * b_bytes + (need + 1) * a_bytes <= budget) {
+        // patches in whole tiles where the taps are outermost
+        const int most = pl->chunk_major ? 4 : 2 * need;
+        if (units <= MAX_B && units * b_bytes + (need + (pl->chunk_major ? 1 : 0)) * a_bytes <=
+                                  budget) {
             pl->resident = 1;
             pl->nb = units;
-            pl->na = std::min(std::min(MAX_A, std::max(4, 2 * need)),
-                              (budget - units * b_bytes) / a_bytes);
+            pl->na = std::min(std::min(MAX_A, most), (budget - units * b_bytes) / a_bytes);
         } else if (c == 1) {
-            // two patches ahead, weights in the rest: at 8 KB a unit, eight
-            // slots covered a third of the L2 latency of a unit's load
             pl->resident = 0;
-            pl->na = std::min(MAX_A, need + 2);
+            pl->na = std::min(std::min(MAX_A, most), (budget - 3 * b_bytes) / a_bytes);
+            if (pl->na < need) return false;
+            if (!pl->chunk_major) pl->na = pl->na / need * need;
             pl->nb = std::min(std::min(units, MAX_B), (budget - pl->na * a_bytes) / b_bytes);
-            if (pl->nb < 3) return false;
         } else {
             continue;
         }
+        if (!pl->chunk_major) pl->na = pl->na / need * need;
         *smem = 128 + pl->na * a_bytes + pl->nb * b_bytes;
         *per_sm = c;
         return true;
@@ -665,7 +705,7 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t st) {
         return cudaErrorNotSupported;
     pl.wbox = pl.slices > 1 && pl.nt <= 128;
     CUtensorMap wmap = map;
-    if (pl.wbox && !weight_map(&wmap, a.w, a.cout, a.cin, pl.nt, pl.kg))
+    if (pl.wbox && !weight_map(&wmap, a.w, a.cout, a.cin, pl.nt, pl.bc * pl.kg))
         return cudaErrorNotSupported;
     // whole slices: every slice gets the same number of CTAs
     int per_slice = std::max(1, sm_count() * per_sm / pl.slices);

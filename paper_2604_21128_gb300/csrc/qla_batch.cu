@@ -244,6 +244,9 @@ struct qla_batch {
     Barrier *d_bar = nullptr;
     double *d_partials = nullptr, *d_energy = nullptr;
     int lane_cols = 0, rows = 0;
+    // the unit list in d_items (0: none), its tiling and the media it is of
+    int list_units = 0, list_rows = 0;
+    std::vector<long long> list_gens;
     long long budget = 1LL << 31;
     int skip_block = -1;
     long long launches = 0;
@@ -274,18 +277,19 @@ bool lattice_ok(int nx, int ny, int planes) {
            offsets32_ok(size_t(planes), padded_plane(nx, ny));
 }
 
-// Work-list capacity (rows per item >= 32): items of the two-column
+// Work-list capacity (rows per item >= MIN_ROWS): items of the two-column
 // layout, or units of the plateau split (three per 120-column item).
+constexpr int MIN_ROWS = 16;
 size_t items_of(int count, const int *nx, const int *ny) {
     size_t items = 0;
     for (int k = 0; k < count; ++k)
-        items += size_t((nx[k] + 55) / 56) * size_t((ny[k] + 31) / 32);
+        items += size_t((nx[k] + 55) / 56) * size_t((ny[k] + MIN_ROWS - 1) / MIN_ROWS);
     return items;
 }
 size_t units_of(int count, const int *nx, const int *ny) {
     size_t units = 0;
     for (int k = 0; k < count; ++k)
-        units += 3 * size_t((nx[k] + PWOUT - 1) / PWOUT) * size_t((ny[k] + 31) / 32);
+        units += 3 * size_t((nx[k] + PWOUT - 1) / PWOUT) * size_t((ny[k] + MIN_ROWS - 1) / MIN_ROWS);
     return units;
 }
 size_t list_bytes(int count, const int *nx, const int *ny) {
@@ -365,19 +369,41 @@ void interleave(const std::vector<std::vector<E>> &per, std::vector<E> &out) {
     }
 }
 
+// Rows per item without a tuning: the tallest segments of up to `most` rows
+// that still give three windows of `wout` columns per resident warp slot
+// (4 blocks of WARPS warps per SM), at least MIN_ROWS.  Tall segments
+// recompute fewer halo rows; with too few items the warps that get one more
+// than others set the step's time, and with less than one each its latency.
+// Measured per step: 24 lattices of sides 512-2048 307 us at 48 rows (three
+// items per slot) against 376 us at 128 and 314 us at 64 or 32; 256 such
+// lattices equal at 64 and 128 rows (six to twelve items per slot), 8% slower
+// at 256.
+int auto_rows(const qla_batch *b, int wout, int most) {
+    const long long slots = 4LL * WARPS * b->num_sms;
+    for (int rows = most; rows > MIN_ROWS; rows -= 16) {
+        long long items = 0;
+        for (const qla_ctx *c : b->inst)
+            items += (long long)((c->nx + wout - 1) / wout) * ((c->ny + rows - 1) / rows);
+        if (items >= 3 * slots) return rows;
+    }
+    return MIN_ROWS;
+}
+
 // Units of the plateau-split kernel (segments of `seg` rows, capped at each
 // lattice's height): every instance's items classified on the GPU (into the
 // batch's work list, which the units then replace; the instances' own unit
 // lists belong to their single-lattice steps), then the other items' units
 // of all instances, interleaved, followed by the plateau units, interleaved.
+// A list stays as long as the tiling and every instance's medium do.
 qla_status build_units(qla_batch *b, int rows, int *n_units, std::vector<BatchInst> &hinst) {
+    std::vector<long long> gens(b->count);
+    for (int k = 0; k < b->count; ++k) gens[k] = b->inst[k]->medium_gen;
+    const bool keep = b->list_units > 0 && b->list_rows == rows && b->list_gens == gens;
     std::vector<int> segs(b->count), nwx(b->count), nitems(b->count);
     std::vector<size_t> at(b->count + 1, 0);
     for (int k = 0; k < b->count; ++k) {
         qla_ctx *c = b->inst[k];
-        // 128-row segments by default (256 instances of sides 512-2048:
-        // 1.64e11 site-updates/s at 64 or 128 rows, 1.52e11 at 256)
-        int seg = rows > 0 ? rows : 128;
+        int seg = rows > 0 ? rows : auto_rows(b, PWOUT, 128);
         seg = (seg + 3) / 4 * 4;
         if (seg > c->ny) seg = (c->ny + 3) / 4 * 4;
         segs[k] = seg;
@@ -385,39 +411,46 @@ qla_status build_units(qla_batch *b, int rows, int *n_units, std::vector<BatchIn
         nitems[k] = nwx[k] * ((c->ny + seg - 1) / seg);
         at[k + 1] = at[k] + size_t(nitems[k]);
     }
-    if (at[b->count] > b->units_cap)   // classes take 4 of a unit's 32 bytes
-        return bfail(b, QLA_EINVAL, "qla_batch: %zu items exceed the workspace's %zu",
-                     at[b->count], b->units_cap);
-    int *cls_dev = reinterpret_cast<int *>(b->d_items);
-    for (int k = 0; k < b->count; ++k) {
-        qla_ctx *c = b->inst[k];
-        k_classify_items<<<(nitems[k] + WARPS - 1) / WARPS, 32 * WARPS, 0, b->stream>>>(
-            c->midx, c->nx, c->ny, c->pitch, segs[k], nwx[k], nitems[k], cls_dev + at[k]);
-        BCUDA(b, cudaGetLastError(), "qla_batch: classify");
+    if (!keep) {
+        b->list_units = 0;
+        if (at[b->count] > b->units_cap)   // classes take 4 of a unit's 32 bytes
+            return bfail(b, QLA_EINVAL, "qla_batch: %zu items exceed the workspace's %zu",
+                         at[b->count], b->units_cap);
+        int *cls_dev = reinterpret_cast<int *>(b->d_items);
+        for (int k = 0; k < b->count; ++k) {
+            qla_ctx *c = b->inst[k];
+            k_classify_items<<<(nitems[k] + WARPS - 1) / WARPS, 32 * WARPS, 0, b->stream>>>(
+                c->midx, c->nx, c->ny, c->pitch, segs[k], nwx[k], nitems[k], cls_dev + at[k]);
+            BCUDA(b, cudaGetLastError(), "qla_batch: classify");
+        }
+        std::vector<int> all(at[b->count]);
+        BCUDA(b, cudaMemcpyAsync(all.data(), cls_dev, all.size() * 4, cudaMemcpyDeviceToHost,
+                                 b->stream), "qla_batch: classes");
+        BCUDA(b, cudaStreamSynchronize(b->stream), "qla_batch: classes");
+        std::vector<std::vector<int>> cls(b->count);
+        for (int k = 0; k < b->count; ++k)
+            cls[k].assign(all.begin() + at[k], all.begin() + at[k + 1]);
+        std::vector<std::vector<BatchUnit>> other(b->count), plat(b->count);
+        for (int k = 0; k < b->count; ++k) {
+            qla_ctx *c = b->inst[k];
+            std::vector<int4> o, p;
+            plateau_units(cls[k], c->nx, c->ny, segs[k], o, p);
+            for (const int4 &u : o) other[k].push_back(BatchUnit{u, k, 0, 0, 0});
+            for (const int4 &u : p) plat[k].push_back(BatchUnit{u, k, 0, 0, 0});
+        }
+        std::vector<BatchUnit> list;
+        interleave(other, list);
+        interleave(plat, list);
+        if (list.size() > b->units_cap)
+            return bfail(b, QLA_EINVAL, "qla_batch: %zu units exceed the workspace's %zu",
+                         list.size(), b->units_cap);
+        BCUDA(b, cudaMemcpyAsync(b->d_items, list.data(), list.size() * sizeof(BatchUnit),
+                                 cudaMemcpyHostToDevice, b->stream), "qla_batch: units");
+        BCUDA(b, cudaStreamSynchronize(b->stream), "qla_batch: units");
+        b->list_units = int(list.size());
+        b->list_rows = rows;
+        b->list_gens = gens;
     }
-    std::vector<int> all(at[b->count]);
-    BCUDA(b, cudaMemcpyAsync(all.data(), cls_dev, all.size() * 4, cudaMemcpyDeviceToHost,
-                             b->stream), "qla_batch: classes");
-    BCUDA(b, cudaStreamSynchronize(b->stream), "qla_batch: classes");
-    std::vector<std::vector<int>> cls(b->count);
-    for (int k = 0; k < b->count; ++k)
-        cls[k].assign(all.begin() + at[k], all.begin() + at[k + 1]);
-    std::vector<std::vector<BatchUnit>> other(b->count), plat(b->count);
-    for (int k = 0; k < b->count; ++k) {
-        qla_ctx *c = b->inst[k];
-        std::vector<int4> o, p;
-        plateau_units(cls[k], c->nx, c->ny, segs[k], o, p);
-        for (const int4 &u : o) other[k].push_back(BatchUnit{u, k, 0, 0, 0});
-        for (const int4 &u : p) plat[k].push_back(BatchUnit{u, k, 0, 0, 0});
-    }
-    std::vector<BatchUnit> list;
-    interleave(other, list);
-    interleave(plat, list);
-    if (list.size() > b->units_cap)
-        return bfail(b, QLA_EINVAL, "qla_batch: %zu units exceed the workspace's %zu",
-                     list.size(), b->units_cap);
-    BCUDA(b, cudaMemcpyAsync(b->d_items, list.data(), list.size() * sizeof(BatchUnit),
-                             cudaMemcpyHostToDevice, b->stream), "qla_batch: units");
     hinst.resize(b->count);
     for (int k = 0; k < b->count; ++k) {
         qla_ctx *c = b->inst[k];
@@ -439,7 +472,7 @@ qla_status build_units(qla_batch *b, int rows, int *n_units, std::vector<BatchIn
     BCUDA(b, cudaMemcpyAsync(b->d_insts, hinst.data(), hinst.size() * sizeof(BatchInst),
                              cudaMemcpyHostToDevice, b->stream), "qla_batch: instances");
     BCUDA(b, cudaStreamSynchronize(b->stream), "qla_batch: upload");
-    *n_units = int(list.size());
+    *n_units = b->list_units;
     return QLA_OK;
 }
 
@@ -448,11 +481,12 @@ qla_status build_items(qla_batch *b, int lx, int rows, int *n_items,
                        std::vector<BatchInst> &hinst) {
     if (kernels(b, lx).plateau) return build_units(b, rows, n_items, hinst);
     const int wout = window_out(lx);
+    b->list_units = 0;   // the items replace a unit list
     std::vector<BatchItem> items;
     hinst.resize(b->count);
     for (int k = 0; k < b->count; ++k) {
         qla_ctx *c = b->inst[k];
-        int seg = rows > 0 ? rows : 256;
+        int seg = rows > 0 ? rows : auto_rows(b, wout, 256);
         seg = (seg + 3) / 4 * 4;
         if (seg > c->ny) seg = (c->ny + 3) / 4 * 4;
         const int n_wx = (c->nx + wout - 1) / wout, n_wy = (c->ny + seg - 1) / seg;
@@ -492,7 +526,7 @@ qla_status build_items(qla_batch *b, int lx, int rows, int *n_items,
     }
     if (mixed.size() > b->items_cap)
         return bfail(b, QLA_EINVAL, "qla_batch: %zu work items exceed the workspace's %zu "
-                     "(rows per item below 32?)", mixed.size(), b->items_cap);
+                     "(rows per item below %d?)", mixed.size(), b->items_cap, MIN_ROWS);
     BCUDA(b, cudaMemcpyAsync(b->d_items, mixed.data(), mixed.size() * sizeof(BatchItem),
                              cudaMemcpyHostToDevice, b->stream), "qla_batch: items");
     BCUDA(b, cudaMemcpyAsync(b->d_insts, hinst.data(), hinst.size() * sizeof(BatchInst),

@@ -647,8 +647,11 @@ template <typename T, int VM, int PD>
 __global__ void __launch_bounds__(128)
 k3_zcol(const T *__restrict__ in, T *__restrict__ out, const uint32_t *__restrict__ idx3,
         const MedRec<T> *__restrict__ rec, const V3<T> *__restrict__ rv, int nx, int ny, int nz,
-        int pitch, size_t plane_elems, int seg) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        int pitch, size_t plane_elems, int seg, int nseg) {
+    // the segments of a group of columns are consecutive blocks: the planes
+    // two of them read come from L2
+    const int sz = int(blockIdx.x % unsigned(nseg));
+    const long long t = (long long)(blockIdx.x / unsigned(nseg)) * blockDim.x + threadIdx.x;
     // threads past the last column have nothing to do (no barrier follows)
     if (t >= (long long)nx * ny) return;
     ZCol<T, VM, PD> m;
@@ -662,7 +665,7 @@ k3_zcol(const T *__restrict__ in, T *__restrict__ out, const uint32_t *__restric
     m.zstride = size_t(ny) * pitch;
     m.plane_elems = plane_elems;
     m.nz = nz;
-    const int z_lo = int(blockIdx.y) * seg, z_hi = min(nz, z_lo + seg);
+    const int z_lo = sz * seg, z_hi = min(nz, z_lo + seg);
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
         m.dring[l][0] = m.dring[l][1] = T(0);
@@ -695,6 +698,26 @@ bool slices_ok(int nx, int ny, size_t plane_elems) {
     return nx % 2 == 0 && nx >= 64 && ny >= 8 && 6 * (unsigned long long)plane_elems < (1ull << 32);
 }
 
+// Segment length of an axis of `len` for launches of `per_seg` work items per
+// segment over `slots` resident ones: whole waves times a segment with its
+// eight halo rows or planes, in steps of four, at least min_seg.  (192 x 160
+// x 128 FP32, us per step, of which the rest of the step 104: rows 32 116, 40
+// 104, 56 110, 80 125; column planes 16 99, 32 99, 44 114, 64 92, 128 154.)
+int pick_waves(int len, long long per_seg, long long slots, int min_seg) {
+    int best = len;
+    long long best_cost = -1;
+    for (int n = 1; n <= (len + min_seg - 1) / min_seg; ++n) {
+        const int seg = std::max(min_seg, ((len + n - 1) / n + 3) / 4 * 4);
+        const long long items = per_seg * ((len + seg - 1) / seg);
+        const long long cost = (items + slots - 1) / slots * (seg + 2 * HALO3);
+        if (best_cost < 0 || cost < best_cost) {
+            best = seg;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 // Launch 1 of the slices step for the plane set PS.
 template <typename T, int PS>
 cudaError_t slices_launch(const void *in, void *out, const uint32_t *idx3, const void *rec,
@@ -714,20 +737,16 @@ cudaError_t slices_launch(const void *in, void *out, const uint32_t *idx3, const
         if (per_sm < 1) per_sm = 1;
     });
     if (attr != cudaSuccess) return attr;
-    // launch 1: items of 64-column windows (56 stored) x row segments x slices,
-    // about two per resident warp slot
+    // launch 1: items of 64-column windows (56 stored) x row segments x slices
     const int n_wx = (nx + 55) / 56;
-    const long long resident = (long long)per_sm * march::WARPS * num_sms;
-    long long n_wy = 2 * resident / ((long long)n_wx * nz);
-    if (n_wy < 1) n_wy = 1;
-    int seg_h = int((ny + n_wy - 1) / n_wy);
-    seg_h = seg_h < 32 ? 32 : (seg_h + 3) / 4 * 4;
-    n_wy = (ny + seg_h - 1) / seg_h;
+    const int seg_h = pick_waves(ny, (long long)n_wx * nz,
+                                 (long long)per_sm * march::WARPS * num_sms, 32);
+    const int n_wy = (ny + seg_h - 1) / seg_h;
     const long long n_items = (long long)n_wx * n_wy * nz;
     const long long blocks = (n_items + march::WARPS - 1) / march::WARPS;
     k1<<<unsigned(blocks), 32 * march::WARPS, smem, st>>>(
         static_cast<const T *>(in), static_cast<T *>(out), idx3,
-        static_cast<const MedRec<T> *>(rec), nx, ny, pitch, plane_elems, seg_h, n_wx, int(n_wy),
+        static_cast<const MedRec<T> *>(rec), nx, ny, pitch, plane_elems, seg_h, n_wx, n_wy,
         n_items);
     return cudaGetLastError();
 }
@@ -753,21 +772,27 @@ cudaError_t slices_t(const void *in, void *out, const uint32_t *idx3, const void
         e = slices_launch<T, 6>(in, out, idx3, rec, nx, ny, nz, pitch, plane_elems, num_sms, st);
     }
     if (e != cudaSuccess) return e;
-    // launch 2: one thread per column, z segments for about two waves of
-    // 128-thread blocks (at least 16 planes each)
+    // launch 2: one thread per column and z segment.  FP32 loads four planes
+    // ahead (3.5% faster than one at 256^3); FP64 is bound by its FMA pipe and
+    // loads one ahead; double-single two
+    constexpr int PD = sizeof(T) == 4 ? 4 : std::is_same<T, dsf>::value ? 2 : 1;
+    auto k2 = k3_zcol<T, VM, PD>;
+    struct Occ { cudaError_t err; int per_sm; };
+    static const Occ occ = [&] {
+        Occ o{cudaSuccess, 1};
+        o.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.per_sm, k2, 128, 0);
+        if (o.per_sm < 1) o.per_sm = 1;
+        return o;
+    }();
+    if (occ.err != cudaSuccess) return occ.err;
     const long long cols = (long long)nx * ny;
     const long long cblocks = (cols + 127) / 128;
-    int nseg = int((2LL * 8 * num_sms + cblocks - 1) / cblocks);
-    if (nseg < 1) nseg = 1;
-    int seg = (nz + nseg - 1) / nseg;
-    if (seg < 16) seg = 16;
-    nseg = (nz + seg - 1) / seg;
-    // FP32 loads four planes ahead (3.5% faster than one at 256^3); FP64 is
-    // bound by its FMA pipe and loads one ahead; double-single two
-    k3_zcol<T, VM, sizeof(T) == 4 ? 4 : (std::is_same<T, dsf>::value ? 2 : 1)><<<dim3(unsigned(cblocks), nseg), 128, 0, st>>>(
+    const int seg = pick_waves(nz, cblocks, (long long)occ.per_sm * num_sms, 16);
+    const int nseg = (nz + seg - 1) / seg;
+    k2<<<unsigned(cblocks * nseg), 128, 0, st>>>(
         static_cast<const T *>(out), static_cast<T *>(const_cast<void *>(in)), idx3,
         static_cast<const MedRec<T> *>(rec), static_cast<const V3<T> *>(rv), nx, ny, nz, pitch,
-        plane_elems, seg);
+        plane_elems, seg, nseg);
     return cudaGetLastError();
 }
 

@@ -69,10 +69,10 @@ Layout layout_for(int nx, int ny, int prec, unsigned flags) {
     if ((flags & QLA_DOUBLE_SINGLE) && prec == QLA_FP64) {
         L.dstable = off; off += align256((UNIFORM_SLOTS + sites) * sizeof(MedRec<dsf>));
     }
-    // FP32 E_z: the plateau-split step's unit list (int4 entries): three
-    // units per 120-column window and segment of at least 16 rows
+    // FP32: the plateau-split step's unit list (int4 entries): three units
+    // per 120-column window and segment of at least 16 rows
     L.items = L.items_cap = 0;
-    if (prec == QLA_FP32 && P == 3) {
+    if (prec == QLA_FP32) {
         L.items_cap = 3 * size_t((nx + 119) / 120) * size_t((ny + 15) / 16);
         L.items = off; off += align256(L.items_cap * 16);
     } else if (prec == QLA_FP64 && P == 3 && (flags & QLA_DOUBLE_SINGLE)) {

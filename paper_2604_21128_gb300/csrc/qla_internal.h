@@ -428,7 +428,7 @@ struct Layout {
     size_t n_x, n_y, ttable;  // QLA_ANISOTROPIC only (else 0)
     size_t tile_done;         // TILE_COUNTERS counters
     size_t dstable;           // QLA_DOUBLE_SINGLE only (else 0)
-    size_t items, items_cap;  // FP32 E_z only (else 0): marching work-item list
+    size_t items, items_cap;  // FP32, or double-single E_z (else 0): marching units
     size_t plane_elems;
     int pitch, energy_blocks;
 };

@@ -1,5 +1,5 @@
-// Plateau work units of the E_z marching steps: FP32 (single lattices and
-// batches) and double-single.
+// Plateau work units of the marching steps: FP32 (E_z lattices and batches,
+// and the two triples of six-plane lattices) and double-single E_z.
 //
 // In the workloads' media most sites sit on plateaus of n on which every
 // site's four neighbours carry its n: those share one record (see MedRec),
@@ -34,8 +34,9 @@ __host__ __device__ inline int4 plateau_unit(int x_out, int w_out, int rec, int 
 }
 
 // Run unit u of a lattice (arrays in/out/midx/table of its size and pitch);
-// smem: this warp's staging ring (room for the four-column ring).
-template <int VM, bool VIN>
+// smem: this warp's staging ring (room for the four-column ring).  P: the
+// E_z storage, or one triple of a six-plane one.
+template <int VM, bool VIN, int P = 3>
 __device__ __forceinline__ void run_plateau_unit(const float *in, float *out, const uint32_t *midx,
                                                  const MedRec<float> *table, int nx, int ny,
                                                  int pitch, uint32_t plane, const int4 &u,
@@ -43,7 +44,7 @@ __device__ __forceinline__ void run_plateau_unit(const float *in, float *out, co
     const int w_out = u.y & 0xff, rec = (u.y >> 8) - 1;
     if (w_out == 0) return;
     if (rec >= 0) {
-        using M = March<float, 3, 4, VM, VIN, true>;
+        using M = March<float, P, 4, VM, VIN, true>;
         M m;
         m.in = in;
         m.out = out;
@@ -56,7 +57,7 @@ __device__ __forceinline__ void run_plateau_unit(const float *in, float *out, co
         m.set_uniform(__ldg(&table[rec].c));
         m.run_unit(nx, ny, u.x, w_out, u.z, u.w, reinterpret_cast<typename M::Slot *>(smem));
     } else {
-        using M = March<float, 3, 2, VM, VIN, false>;
+        using M = March<float, P, 2, VM, VIN, false>;
         M m;
         m.in = in;
         m.out = out;

@@ -114,6 +114,33 @@ k_step_march_split(const float *__restrict__ in, float *__restrict__ out,
                               smem_raw + warp * plateau_ring_bytes<VM, VIN>());
 }
 
+// The plateau split of a six-plane step: the two decoupled triples (q2, q3,
+// q4) and (q0, q1, q5) run the same unit list, each on its own planes, as
+// blockIdx.y 0 and 1 of one launch.  A six-plane march has no registers for
+// four columns per lane, and its 64-column windows recompute an eighth of
+// their columns; a triple's plateau units recompute a sixteenth and carry
+// neither record ring nor lookups.  Units where n varies cost about what half
+// a six-plane item does.  4096^2 with an ellipse, us per step: 287 for the
+// six-plane march, 255 split.
+template <int VM, bool VIN>
+__global__ void __launch_bounds__(32 * WARPS, 4)
+k_step_march_split6(const float *__restrict__ in, float *__restrict__ out,
+                    const uint32_t *__restrict__ midx, const MedRec<float> *__restrict__ table,
+                    int nx, int ny, int pitch, size_t plane, const int4 *__restrict__ units,
+                    int n_units) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5;
+    const int li = int(blockIdx.x) * WARPS + warp;
+    if (li >= n_units) return;   // the whole warp: units are per warp
+    unsigned char *ring = smem_raw + warp * plateau_ring_bytes<VM, VIN>();
+    if (blockIdx.y == 0)
+        run_plateau_unit<VM, VIN, P_TE6>(in, out, midx, table, nx, ny, pitch, uint32_t(plane),
+                                         units[li], ring);
+    else
+        run_plateau_unit<VM, VIN, P_TM6>(in, out, midx, table, nx, ny, pitch, uint32_t(plane),
+                                         units[li], ring);
+}
+
 // Dataflow steps of the plateau split (see flow_wait): n_steps steps of
 // the unit list in one persistent launch, buffers a (the input of even
 // steps) and b.  Blocks take four consecutive units w .. w + 3 (w = s *
@@ -513,6 +540,45 @@ cudaError_t launch_split(qla_ctx *c, const void *in, void *out) {
     return cudaGetLastError();
 }
 
+template <int VM, bool VIN>
+cudaError_t launch_split6(qla_ctx *c, const void *in, void *out) {
+    auto kern = k_step_march_split6<VM, VIN>;
+    const size_t smem = plateau_ring_bytes<VM, VIN>() * WARPS;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (attr != cudaSuccess) return attr;
+    const auto &u = c->uplan;
+    kern<<<dim3(unsigned((u.n_list + WARPS - 1) / WARPS), 2), 32 * WARPS, smem, c->stream>>>(
+        static_cast<const float *>(in), static_cast<float *>(out), c->midx,
+        static_cast<const MedRec<float> *>(c->table), c->nx, c->ny, c->pitch, c->plane_elems,
+        reinterpret_cast<const int4 *>(c->items), u.n_list);
+    return cudaGetLastError();
+}
+
+// Segment height of the six-plane split: whole waves of units (both triples)
+// over the resident warp slots, each a segment with its eight halo rows, plus
+// half a segment for the tail; rows a multiple of 4, at least 16.  0 (no
+// split) below two and a half waves of 32-row units: with fewer, the units'
+// latency counts and the six-plane march, which has both triples' rotations
+// in flight per warp, is faster (us per step, march against split: 2048^2 89
+// / 102, 1536^2 69 / 64, 3000 x 1100 90 / 87 at 32 rows, 4096^2 287 / 255).
+int split6_segment(const qla_ctx *c) {
+    const long long per = 2LL * ((c->nx + PWOUT - 1) / PWOUT);
+    const long long slots = 4LL * WARPS * c->num_sms;
+    if (2 * per * ((c->ny + 31) / 32) < 5 * slots) return 0;
+    int best = 16;
+    long long best_cost = -1;
+    for (int seg = 16; seg <= 256; seg += 4) {
+        const long long units = per * ((c->ny + seg - 1) / seg);
+        const long long cost = (2 * ((units + slots - 1) / slots) + 1) * (seg + 2 * LAG);
+        if (best_cost < 0 || cost < best_cost) {
+            best = seg;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 template <typename T, int P, int LX, int VM, bool VIN>
 cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
     using V = Variant<T, P, LX, VM, VIN>;
@@ -574,6 +640,19 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
             }
             if (u.gen == c->medium_gen && u.seg == pseg && u.n_uniform > 0)
                 return launch_split<VM, VIN>(c, in, out);
+        }
+    }
+    if constexpr (std::is_same<T, float>::value && P == 6) {
+        if (c->items && c->step_kernel != QLA_KERNEL_MARCH_PLAIN && c->nx % 4 == 0 &&
+            c->nx >= PW) {
+            const int sseg = c->march_seg > 0 ? std::max(16, seg) : split6_segment(c);
+            if (sseg > 0) {
+                const cudaError_t e = ensure_plateau_plan(c, sseg, false);
+                if (e != cudaSuccess) return e;
+            }
+            const auto &u = c->uplan;
+            if (sseg > 0 && u.gen == c->medium_gen && u.seg == sseg && u.n_uniform > 0)
+                return launch_split6<VM, VIN>(c, in, out);
         }
     }
     if constexpr (std::is_same<T, dsf>::value && P == 3 && LX == 2) {

@@ -490,7 +490,7 @@ cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done
     // lattices that the plateau split takes keep it for calls of up to three
     // steps, which are short either way: qla_march_plan then has a plan to
     // describe from the first call on
-    if (c->items && n_steps < 4 && march_supported(c) && c->nx % 4 == 0 &&
+    if (c->items && c->P == 3 && n_steps < 4 && march_supported(c) && c->nx % 4 == 0 &&
         size_t(c->nx) * c->ny >= (size_t(1) << 18))
         return cudaSuccess;
     const long long n = std::min<long long>(n_steps, 1LL << 24);

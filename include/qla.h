@@ -556,7 +556,7 @@ qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_bf16, int B,
                                 void *cuda_stream);
 
 /* Test hook for the bounded waits: while on is non-zero, one CTA of every
- * gather-form tensor-core convolution waits for an mbarrier phase that never
+ * tensor-core convolution waits for an mbarrier phase that never
  * completes, gives up after 2 s of wall time, skips its output and raises
  * the error flag, so surr_conv3x3_raw returns QLA_ETIMEOUT (and the
  * network's next synchronising call would).  No fault and no hang: the other

@@ -699,11 +699,18 @@ bool slices_ok(int nx, int ny, size_t plane_elems) {
 }
 
 // Segment length of an axis of `len` for launches of `per_seg` work items per
-// segment over `slots` resident ones: whole waves times a segment with its
-// eight halo rows or planes, in steps of four, at least min_seg.  (192 x 160
-// x 128 FP32, us per step, of which the rest of the step 104: rows 32 116, 40
-// 104, 56 110, 80 125; column planes 16 99, 32 99, 44 114, 64 92, 128 154.)
-int pick_waves(int len, long long per_seg, long long slots, int min_seg) {
+// segment over `slots` resident ones, at least min_seg and a multiple of 4.
+// State beyond the L2 (big): whole waves times a segment with its eight halo
+// rows or planes, which are read again from memory (192 x 160 x 128 FP32, us
+// of the launch: rows 32 116, 40 104, 56 110, 80 125; column planes 16 99, 32
+// 99, 44 114, 64 92, 128 154).  State in the L2: about two waves; the halo is
+// cheap there and more items in flight hide more latency (66 x 174 x 180: the
+// first rule 2% slower).
+int pick_segment3(int len, long long per_seg, long long slots, int min_seg, bool big) {
+    if (!big) {
+        const long long n = std::max(1LL, 2 * slots / per_seg);
+        return std::max(min_seg, (int((len + n - 1) / n) + 3) / 4 * 4);
+    }
     int best = len;
     long long best_cost = -1;
     for (int n = 1; n <= (len + min_seg - 1) / min_seg; ++n) {
@@ -716,6 +723,11 @@ int pick_waves(int len, long long per_seg, long long slots, int min_seg) {
         }
     }
     return best;
+}
+// Both state buffers exceed the 126 MB L2.
+template <typename T>
+bool beyond_l2(size_t plane_elems) {
+    return 12.0 * double(plane_elems) * sizeof(T) > 126e6;
 }
 
 // Launch 1 of the slices step for the plane set PS.
@@ -739,8 +751,9 @@ cudaError_t slices_launch(const void *in, void *out, const uint32_t *idx3, const
     if (attr != cudaSuccess) return attr;
     // launch 1: items of 64-column windows (56 stored) x row segments x slices
     const int n_wx = (nx + 55) / 56;
-    const int seg_h = pick_waves(ny, (long long)n_wx * nz,
-                                 (long long)per_sm * march::WARPS * num_sms, 32);
+    const int seg_h = pick_segment3(ny, (long long)n_wx * nz,
+                                    (long long)per_sm * march::WARPS * num_sms, 32,
+                                    beyond_l2<T>(plane_elems));
     const int n_wy = (ny + seg_h - 1) / seg_h;
     const long long n_items = (long long)n_wx * n_wy * nz;
     const long long blocks = (n_items + march::WARPS - 1) / march::WARPS;
@@ -787,7 +800,10 @@ cudaError_t slices_t(const void *in, void *out, const uint32_t *idx3, const void
     if (occ.err != cudaSuccess) return occ.err;
     const long long cols = (long long)nx * ny;
     const long long cblocks = (cols + 127) / 128;
-    const int seg = pick_waves(nz, cblocks, (long long)occ.per_sm * num_sms, 16);
+    // (two waves of eight 128-thread blocks per SM where the state fits the L2)
+    const bool big = beyond_l2<T>(plane_elems);
+    const int seg = pick_segment3(nz, cblocks, (long long)(big ? occ.per_sm : 8) * num_sms, 16,
+                                  big);
     const int nseg = (nz + seg - 1) / seg;
     k2<<<unsigned(cblocks * nseg), 128, 0, st>>>(
         static_cast<const T *>(out), static_cast<T *>(const_cast<void *>(in)), idx3,

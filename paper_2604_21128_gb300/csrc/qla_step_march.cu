@@ -646,11 +646,17 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
         if (c->items && c->step_kernel != QLA_KERNEL_MARCH_PLAIN && c->nx % 4 == 0 &&
             c->nx >= PW) {
             const int sseg = c->march_seg > 0 ? std::max(16, seg) : split6_segment(c);
-            if (sseg > 0) {
-                const cudaError_t e = ensure_plateau_plan(c, sseg, false);
+            const auto &u = c->uplan;
+            // building the plan waits for the stream: not inside a capture,
+            // where the six-plane march needs no plan
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            const bool have = u.gen == c->medium_gen && u.seg == sseg;
+            if (sseg > 0 && !have) {
+                cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+                if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+                    e = ensure_plateau_plan(c, sseg, false);
                 if (e != cudaSuccess) return e;
             }
-            const auto &u = c->uplan;
             if (sseg > 0 && u.gen == c->medium_gen && u.seg == sseg && u.n_uniform > 0)
                 return launch_split6<VM, VIN>(c, in, out);
         }

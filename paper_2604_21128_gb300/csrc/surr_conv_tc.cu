@@ -30,9 +30,9 @@
 //
 // What bounds it: for N = 16 or 32 the operand reads from shared memory (an
 // MMA reads 4 KB of pixels for 16 K multiply-adds per output channel), for
-// wider N the tensor pipe; see conv_cost.  Batch 8 at 256^2, us per layer
-// (row patches and per-tap gathers before): 45 27 36 43 43 83 120 95 93 59
-// before.
+// wider N the tensor pipe (conv_cost), and the epilogues.  Batch 8 at 256^2, us per
+// layer: 30 18 18 17 21 26 42 39 34 24; with row patches and per-tap gathers, and
+// separate pooling and upsampling, 53 32 41 47 47 90 131 113 93 71.
 //
 // Every wait on an mbarrier gives up after WAIT_NS of %globaltimer time; a CTA
 // that gives up raises conv_tc_error, lets its copies in flight land, frees

@@ -493,6 +493,8 @@ cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done
 // Whether an automatic context's steps go to the tile kernel although the
 // marching kernel takes its lattice.
 bool tile_steps_pay(const qla_ctx *c);
+// An FP64 marching step's time in item rows (see pick_segment64).
+double march64_rows(const qla_ctx *c);
 // Clears the wait flag unless launches since its last read may have raised it.
 cudaError_t reset_wait_flag(qla_ctx *c);
 bool march_supported(const qla_ctx *c);

@@ -257,6 +257,34 @@ inline int pick_segment(int ny, int n_wx, long long resident_warps, int min_seg 
     return best;
 }
 
+// Segment height of the FP64 march.  It is bound by the FP64 pipe, which one
+// warp per scheduler keeps busy for 70% (a 40-row item takes 168 us alone) and
+// two for 78%, so a step's time goes by whole waves of four items per SM: one
+// takes a segment's rows (with eight halo rows), w of them 0.9 w as long (six
+// planes 0.82 w).  The height that gives the least of that, at least 32 rows,
+// a multiple of 4.  *cost: it, in rows.  Measured, us per step, against about
+// two items per SM and scheduler whatever the remainder: E_z 1152^2 301 ->
+// 217, 1536^2 449 -> 332, 2560^2 1010 -> 806, 3072^2 1512 -> 1103; six planes
+// 2048^2 1039 -> 970, 3072^2 2275 -> 1985.
+int pick_segment64(int ny, int n_wx, int num_sms, bool te, double *cost) {
+    const long long slots = 4LL * num_sms;
+    const double many = te ? 0.9 : 0.82;
+    int best = 32;
+    double best_cost = -1.0;
+    for (int n = 1; n <= (ny + 31) / 32; ++n) {
+        const int seg = std::max(32, ((ny + n - 1) / n + 3) / 4 * 4);
+        const long long items = (long long)n_wx * ((ny + seg - 1) / seg);
+        const long long waves = (items + slots - 1) / slots;
+        const double t = (waves == 1 ? 1.0 : many * double(waves)) * (seg + 2 * LAG);
+        if (best_cost < 0.0 || t < best_cost) {
+            best = seg;
+            best_cost = t;
+        }
+    }
+    if (cost) *cost = best_cost;
+    return best;
+}
+
 // Kernel, staged-row size and stored columns per window of a variant; LX = 1
 // selects the packed-pair kernel (FP32 E_z).
 template <typename T, int P, int LX, int VM, bool VIN> struct Variant {
@@ -601,13 +629,9 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
     const int n_wx = (c->nx + WOUT - 1) / WOUT;
     int seg = c->march_seg;
     if (seg <= 0) {
-        long long resident = (long long)blocks_per_sm * WARPS * c->num_sms;
-        // FP64 E_z is bound by the FP64 pipe, which few warps keep busy, while
-        // every segment re-reads 8 rows: half an item per resident warp slot
-        // measured best (8192^2: 1024-row segments 8.6e9 site-updates/s
-        // against 8.4e9 at 256; 4096^2: 256 rows 8.4e9 against 7.7e9 at 64)
-        if (std::is_same<T, double>::value && P == 3) resident /= 4;
-        seg = pick_segment(c->ny, n_wx, resident);
+        seg = std::is_same<T, double>::value
+                  ? pick_segment64(c->ny, n_wx, c->num_sms, P == 3, nullptr)
+                  : pick_segment(c->ny, n_wx, (long long)blocks_per_sm * WARPS * c->num_sms);
     } else {
         seg = (seg + 3) / 4 * 4;
     }
@@ -765,6 +789,12 @@ cudaError_t launch_step_march(qla_ctx *c, const void *in, void *out, bool vin) {
     case 4: return launch_vm<float, 3, 4>(c, in, out, vin);
     default: return launch_vm<float, 3, 2>(c, in, out, vin);
     }
+}
+
+double march64_rows(const qla_ctx *c) {
+    double rows = 0.0;
+    pick_segment64(c->ny, (c->nx + 55) / 56, c->num_sms, c->P == 3, &rows);
+    return rows;
 }
 
 cudaError_t launch_step_flow(qla_ctx *c, long long n_steps, bool *done) {

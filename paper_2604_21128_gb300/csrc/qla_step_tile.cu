@@ -472,17 +472,18 @@ cudaError_t launch_step_tile(qla_ctx *c, const void *in, void *out, bool vin) {
 }
 
 // Which steps of an automatic context the tile kernel takes from the
-// marching one (measured per step, us, tiles against march):
-//  * FP32 six planes: 1024^2 34.6 / 45.2, 1536^2 69.8 / 69.3
-//  * FP64 E_z: 768^2 98 / 166, 1024^2 176 / 166
-//  * FP64 six planes: 768^2 191 / 312, 1024^2 349 / 323
-//  * FP32 E_z: 768^2 14.5 / 16.6, 1024^2 22.7 / 22.7: resident tiles only
-// (a march has a window's rows in sequence, so lattices with few windows pay
-// its latency whatever their size; tiles pay the halo instead).
+// marching one.  FP32 six planes: 1024^2 34.6 us per step against 45.2,
+// 1536^2 equal.  FP32 E_z: resident tiles only (per-step tiles 768^2 14.5 /
+// 16.6, 1024^2 22.7 / 22.7).  FP64: tiles take 0.165 us per 1000 sites (E_z;
+// 0.325 six planes) at any size, the march 4.2 us (8.1) per row of the items
+// that its schedulers hold one of, whatever the lattice: a march has a
+// window's rows in sequence, so lattices with few windows pay its latency;
+// tiles pay the halo instead (E_z 768^2 98 / 166, 2048^2 655 / 539).
 bool tile_steps_pay(const qla_ctx *c) {
     const size_t sites = size_t(c->nx) * c->ny;
     if (c->prec == QLA_FP32) return c->P == 6 && sites <= (size_t(3) << 19);
-    return sites <= (size_t(7) << 17);
+    const bool te = c->P == 3;
+    return double(sites) * (te ? 0.165e-3 : 0.325e-3) < march64_rows(c) * (te ? 4.2 : 8.1);
 }
 
 cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done) {

@@ -257,25 +257,28 @@ inline int pick_segment(int ny, int n_wx, long long resident_warps, int min_seg 
     return best;
 }
 
-// Segment height of the FP64 march.  It is bound by the FP64 pipe, which one
-// warp per scheduler keeps busy for 70% (a 40-row item takes 168 us alone) and
-// two for 78%, so a step's time goes by whole waves of four items per SM: one
-// takes a segment's rows (with eight halo rows), w of them 0.9 w as long (six
-// planes 0.82 w).  The height that gives the least of that, at least 32 rows,
+// Segment height of the FP64 march.  It is bound by the FP64 pipe, whose cycles
+// one warp per scheduler fills to about 70% by the operation count (a 40-row
+// item takes 168 us alone), so a step's time goes by whole waves of four items
+// per SM: one takes a segment's rows (with eight halo rows), w of them 0.9 w as
+// long (six planes 0.82 w; fitted).  Six planes above 3072^2 keep two items per
+// resident slot, where this rule lost: 4096^2 3535 / 3454, 8192^2 13554 / 12914.
+// The height that gives the least of that, at least 32 rows,
 // a multiple of 4.  *cost: it, in rows.  Measured, us per step, against about
 // two items per SM and scheduler whatever the remainder: E_z 1152^2 301 ->
 // 217, 1536^2 449 -> 332, 2560^2 1010 -> 806, 3072^2 1512 -> 1103; six planes
 // 2048^2 1039 -> 970, 3072^2 2275 -> 1985.
 int pick_segment64(int ny, int n_wx, int num_sms, bool te, double *cost) {
     const long long slots = 4LL * num_sms;
-    const double many = te ? 0.9 : 0.82;
     int best = 32;
     double best_cost = -1.0;
     for (int n = 1; n <= (ny + 31) / 32; ++n) {
         const int seg = std::max(32, ((ny + n - 1) / n + 3) / 4 * 4);
         const long long items = (long long)n_wx * ((ny + seg - 1) / seg);
         const long long waves = (items + slots - 1) / slots;
-        const double t = (waves == 1 ? 1.0 : many * double(waves)) * (seg + 2 * LAG);
+        const double w = double(waves);
+        const double per_wave = waves == 1 ? 1.0 : te ? 0.9 : 0.82;
+        const double t = per_wave * w * (seg + 2 * LAG);
         if (best_cost < 0.0 || t < best_cost) {
             best = seg;
             best_cost = t;
@@ -629,7 +632,7 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
     const int n_wx = (c->nx + WOUT - 1) / WOUT;
     int seg = c->march_seg;
     if (seg <= 0) {
-        seg = std::is_same<T, double>::value
+        seg = std::is_same<T, double>::value && (P == 3 || size_t(c->nx) * c->ny <= (size_t(9) << 20))
                   ? pick_segment64(c->ny, n_wx, c->num_sms, P == 3, nullptr)
                   : pick_segment(c->ny, n_wx, (long long)blocks_per_sm * WARPS * c->num_sms);
     } else {

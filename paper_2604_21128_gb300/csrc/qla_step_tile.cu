@@ -474,8 +474,9 @@ cudaError_t launch_step_tile(qla_ctx *c, const void *in, void *out, bool vin) {
 // Which steps of an automatic context the tile kernel takes from the
 // marching one.  FP32 six planes: 1024^2 34.6 us per step against 45.2,
 // 1536^2 equal.  FP32 E_z: resident tiles only (per-step tiles 768^2 14.5 /
-// 16.6, 1024^2 22.7 / 22.7).  FP64: tiles take 0.165 us per 1000 sites (E_z;
-// 0.325 six planes) at any size, the march 4.2 us (8.1) per row of the items
+// 16.6, 1024^2 22.7 / 22.7).  FP64: tiles take 0.152 to 0.170 us per 1000
+// sites (E_z 1024^2 to 3072^2, compared as 0.165, which leaves 1024^2, 178 /
+// 168, to the march; six planes 0.307 to 0.336, as 0.325), the march 4.2 us (8.1) per row of the items
 // that its schedulers hold one of, whatever the lattice: a march has a
 // window's rows in sequence, so lattices with few windows pay its latency;
 // tiles pay the halo instead (E_z 768^2 98 / 166, 2048^2 655 / 539).

@@ -624,21 +624,10 @@ long long conv_cost(int tiles, int slices, int nt, int sms) {
     return rounds * std::max(32 + nt / 4, nt / 2);
 }
 
-bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
-    const int sms = sm_count();
-    pl->ntx = (a.W + TX - 1) / TX;
-    pl->nty = (a.H + TY - 1) / TY;
-    pl->tiles = a.B * pl->ntx * pl->nty;
-    pl->kg = a.cin % 32 == 0 ? 4 : 2;
-    pl->chunks = a.cin / (8 * pl->kg);
-    pl->nt = 0;
-    for (int nt = 256; nt >= 16; nt /= 2) {
-        if (a.cout % nt || (nt < 32 && a.cout >= 32)) continue;
-        if (!pl->nt || conv_cost(pl->tiles, a.cout / nt, nt, sms) <
-                           conv_cost(pl->tiles, a.cout / pl->nt, pl->nt, sms))
-            pl->nt = nt;
-    }
-    if (!pl->nt) return false;
+// The layout of slices of pl->nt output channels: false where not even three
+// weight units fit beside the patches that have to be resident together (cin
+// = 512 with NT = 256 and the taps outermost, the one such pair).
+bool lay_out(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
     pl->slices = a.cout / pl->nt;
     pl->tcols = std::max(32, 2 * pl->nt);
     // slots of a tile that must be resident together: all of them when the
@@ -683,6 +672,29 @@ bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
         return true;
     }
     return false;
+}
+
+// The cheapest NT (conv_cost; the wider one of equals) that has a layout.
+bool plan_conv(const ConvArgs &a, ConvPlan *pl, int *smem, int *per_sm) {
+    const int sms = sm_count();
+    pl->ntx = (a.W + TX - 1) / TX;
+    pl->nty = (a.H + TY - 1) / TY;
+    pl->tiles = a.B * pl->ntx * pl->nty;
+    pl->kg = a.cin % 32 == 0 ? 4 : 2;
+    pl->chunks = a.cin / (8 * pl->kg);
+    ConvPlan t = *pl;
+    long long best = -1;
+    for (t.nt = 256; t.nt >= 16; t.nt /= 2) {
+        if (a.cout % t.nt || (t.nt < 32 && a.cout >= 32)) continue;
+        const long long cost = conv_cost(t.tiles, a.cout / t.nt, t.nt, sms);
+        int bytes, ctas;
+        if ((best >= 0 && cost >= best) || !lay_out(a, &t, &bytes, &ctas)) continue;
+        best = cost;
+        *pl = t;
+        *smem = bytes;
+        *per_sm = ctas;
+    }
+    return best >= 0;
 }
 
 template <ConvMode MODE>

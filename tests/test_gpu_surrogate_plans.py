@@ -1,0 +1,53 @@
+"""Convolution layouts that the small images of test_gpu_surrogate.py do not
+reach: wide output slices, streamed weights, several tiles per block, against
+FP64 sums on BF16 data."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2604_21128_gb300 import qla
+
+pytestmark = pytest.mark.gpu
+
+
+def bf16(rng, shape, scale=1.0):
+    import torch
+    return torch.tensor(rng.standard_normal(shape) * scale, dtype=torch.float32).bfloat16().cuda()
+
+
+def conv64(x, w):
+    """FP64 periodic convolution on the GPU: x (B, H, W, ci), w (co, 9, ci)."""
+    import torch
+    x, w = x.double(), w.double()
+    out = torch.zeros(x.shape[:3] + (w.shape[0],), dtype=torch.float64, device="cuda")
+    for tap in range(9):
+        shifted = torch.roll(x, (1 - tap // 3, 1 - tap % 3), (1, 2))
+        out += torch.matmul(shifted, w[:, tap].T)
+    return out
+
+
+def conv_raw(x, w):
+    import torch
+    B, H, W, cin = x.shape
+    out = torch.empty((B, H, W, w.shape[0]), dtype=torch.float32, device="cuda")
+    st = qla.load().surr_conv3x3_raw(ctypes.c_void_p(x.data_ptr()), B, H, W, cin,
+                                     ctypes.c_void_p(w.data_ptr()), w.shape[0],
+                                     ctypes.c_void_p(out.data_ptr()), None)
+    return st, out
+
+
+# widths that are no multiple of 128 need a tile's patches resident: with 16
+# of them (cin = 512), 256-channel weight slices do not fit beside
+@pytest.mark.parametrize("B,H,W,cin,cout", [(2, 64, 100, 512, 256), (1, 112, 112, 512, 512),
+                                            (1, 16, 24, 512, 256), (1, 16, 24, 544, 32)])
+def test_wide_inputs_are_taken(B, H, W, cin, cout):
+    import torch
+    rng = np.random.default_rng(cin + cout + W)
+    x, w = bf16(rng, (B, H, W, cin)), bf16(rng, (cout, 9, cin), 0.1)
+    st, out = conv_raw(x, w)
+    assert st == 0
+    want = conv64(x, w)
+    # products of BF16 values are exact; the FP32 accumulation of 9 cin terms
+    # rounds (~sqrt(9 cin) 6e-8 relative)
+    assert float(torch.linalg.norm(out - want) / torch.linalg.norm(want)) <= 1e-5

@@ -482,9 +482,10 @@ void qla_batch_destroy(qla_batch *b);
  * 256; 3x3 periodic convolutions, leaky ReLU 0.1, 2x2 average pooling,
  * nearest 2x upsampling with additive skips; BF16 weights and activations,
  * FP32 accumulation on the tensor cores, FP32 master weights and Adam.
- * The convolutions' device waits are bounded: a wait that runs out makes
- * the next synchronising call (surr_loss_grad, surr_train_step,
- * surr_advance) return QLA_ETIMEOUT.
+ * The device waits of a network's kernels are bounded: one that runs out
+ * raises that network's flag, and its next call that reads the flag
+ * (surr_loss_grad, surr_train_step, surr_advance, surr_get_params) returns
+ * QLA_ETIMEOUT.
  * Inputs per site (features, FP32 [h][w][6]): q2, q3, q4, n - 1.5,
  * 4 dn/dx, 4 dn/dy; output ([h][w][3]): the change of q2, q3, q4.
  * ------------------------------------------------------------------------ */
@@ -518,7 +519,12 @@ qla_status surr_forward(surr_net *n, const float *feat_dev, int B, float *out_de
 qla_status surr_loss_grad(surr_net *n, const float *feat_dev, const float *target_dev, int B,
                           double *loss, float *grad_host);
 
-/* One Adam step (beta 0.9, 0.999, eps 1e-8) at learning rate lr. */
+/* One Adam step (beta 0.9, 0.999, eps 1e-8) at learning rate lr.  Waits for
+ * the loss, not for the backward pass and the update enqueued behind it.  A
+ * step in which a device wait runs out makes no update and is not counted:
+ * QLA_ETIMEOUT from this call if that was before the loss, else from the
+ * network's next call that reads the flag (surr_get_params among them, so
+ * no caller takes the old parameters for updated ones). */
 qla_status surr_train_step(surr_net *n, const float *feat_dev, const float *target_dev, int B,
                            float lr, double *loss);
 
@@ -548,7 +554,10 @@ void surr_destroy(surr_net *n);
  *   out[p][co] = sum_{tap, ci} w[co][tap][ci] in[p + shift(tap)][ci]
  *   dw[co][tap][ci] = sum_p dz[p][co] in[p + shift(tap)][ci]
  * with tap = 3 (dy + 1) + (dx + 1), shifts periodic in y and x; in, w, dz
- * BF16, out and dw FP32; part holds splits * cout * 9 * cin floats. */
+ * BF16, out and dw FP32; part holds splits * cout * 9 * cin floats.  Each call
+ * allocates stream-ordered scratch (cudaMallocAsync) for the network's own
+ * layouts of its operands, frees it and waits for the stream (the second not
+ * while the stream is being captured); QLA_ETIMEOUT if a device wait ran out. */
 qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W, int cin,
                             const void *w_bf16, int cout, float *out_f32, void *cuda_stream);
 qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_bf16, int B, int H, int W,
@@ -556,10 +565,11 @@ qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_bf16, int B,
                                 void *cuda_stream);
 
 /* Test hook for the bounded waits: while on is non-zero, one CTA of every
- * tensor-core convolution waits for an mbarrier phase that never
- * completes, gives up after 2 s of wall time, skips its output and raises
- * the error flag, so surr_conv3x3_raw returns QLA_ETIMEOUT (and the
- * network's next synchronising call would).  No fault and no hang: the other
+ * tensor-core convolution (on = 2: of those with FP32 output, a network's
+ * input gradients) waits for an mbarrier phase that never completes, gives
+ * up after 2 s of wall time and raises the call's or network's flag, unless
+ * that is raised already; surr_conv3x3_raw then returns QLA_ETIMEOUT (and the
+ * network's next call that reads the flag).  No fault and no hang: the other
  * CTAs finish, the stalled one frees its tensor memory and returns. */
 qla_status surr_test_stall_conv(int on);
 

@@ -282,7 +282,7 @@ k_dw_any(const bf16 *__restrict__ dz, const bf16 *__restrict__ in, int H, int W,
 
 template <int MT, int CW, int IW>
 cudaError_t launch_dw(const bf16 *dz, const bf16 *in, int B, const DwGeom &g, int cout, int cin,
-                      int splits, long long per, float *part, cudaStream_t st) {
+                      int splits, long long per, float *part, int *err, cudaStream_t st) {
     auto k = k_dw<MT, CW, IW>;
     const int smem = 128 + DW_STAGES * ((2 * MT * CW * g.z_group() + IW * g.i_group() + 127) / 128 *
                                         128);
@@ -293,9 +293,6 @@ cudaError_t launch_dw(const bf16 *dz, const bf16 *in, int B, const DwGeom &g, in
     if (!blocked_map(&zmap, dz, B, cout, g.h, g.w, false, g.sw, g.sr, 2 * MT * CW) ||
         !blocked_map(&imap, in, B, cin, g.h, g.w, true, g.sw + 2, g.sr + 2, IW))
         return cudaErrorNotSupported;
-    int *err = nullptr;
-    const cudaError_t e = conv_tc_error_ptr(&err);
-    if (e != cudaSuccess) return e;
     k<<<dim3(unsigned(cin / (8 * IW)), unsigned(cout / (16 * MT * CW)), unsigned(splits)),
         32 * CW * IW, smem, st>>>(zmap, imap, g, (long long)B * g.h * g.w, per, cout, cin, part,
                                   err);
@@ -306,11 +303,12 @@ cudaError_t launch_dw(const bf16 *dz, const bf16 *in, int B, const DwGeom &g, in
 // input channels.
 template <int IW>
 cudaError_t launch_dw_co(const bf16 *dz, const bf16 *in, int B, const DwGeom &g, int cout, int cin,
-                         int splits, long long per, float *part, cudaStream_t st) {
+                         int splits, long long per, float *part, int *err, cudaStream_t st) {
     if (cout % 64 == 0 && IW == 4)
-        return launch_dw<2, 2, IW>(dz, in, B, g, cout, cin, splits, per, part, st);
-    if (cout % 32 == 0) return launch_dw<2, 1, IW>(dz, in, B, g, cout, cin, splits, per, part, st);
-    return launch_dw<1, 1, IW>(dz, in, B, g, cout, cin, splits, per, part, st);
+        return launch_dw<2, 2, IW>(dz, in, B, g, cout, cin, splits, per, part, err, st);
+    if (cout % 32 == 0)
+        return launch_dw<2, 1, IW>(dz, in, B, g, cout, cin, splits, per, part, err, st);
+    return launch_dw<1, 1, IW>(dz, in, B, g, cout, cin, splits, per, part, err, st);
 }
 
 // Sums over splits of many arrays: grid.y picks the array.  Many splits of
@@ -542,8 +540,10 @@ __device__ __forceinline__ void put_copies(const LayerParams &l, long long i, fl
 }
 
 __global__ void k_adam(const __grid_constant__ NetParams net, float lr, float b1, float b2,
-                       float eps, float c1, float c2, const int *flag) {
+                       float eps, float c1, float c2, long long step, const int *flag,
+                       long long *applied) {
     if (*flag) return;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *applied = step;
     const LayerParams &l = net.l[blockIdx.y];
     const long long nw = 9LL * l.cout * l.cin, n = nw + l.cout;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
@@ -616,7 +616,7 @@ int weight_grad_splits(int B, int H, int W) {
 }
 
 cudaError_t weight_grad(const bf16 *dz, const bf16 *in, int B, int H, int W, int cout, int cin,
-                        int splits, float *part, cudaStream_t st) {
+                        int splits, float *part, int *err, cudaStream_t st) {
     if (cout % 16 || cin % 16 || splits < 1) return cudaErrorInvalidValue;
     const long long P = (long long)B * H * W;
     long long per = (P + splits - 1) / splits;
@@ -650,9 +650,9 @@ cudaError_t weight_grad(const bf16 *dz, const bf16 *in, int B, int H, int W, int
     };
     int iw = cin % 32 == 0 ? 4 : 2;
     while (iw > 1 && 2 * ctas(iw) <= sms) iw /= 2;
-    if (iw == 4) return launch_dw_co<4>(dz, in, B, g, cout, cin, splits, per, part, st);
-    if (iw == 2) return launch_dw_co<2>(dz, in, B, g, cout, cin, splits, per, part, st);
-    return launch_dw_co<1>(dz, in, B, g, cout, cin, splits, per, part, st);
+    if (iw == 4) return launch_dw_co<4>(dz, in, B, g, cout, cin, splits, per, part, err, st);
+    if (iw == 2) return launch_dw_co<2>(dz, in, B, g, cout, cin, splits, per, part, err, st);
+    return launch_dw_co<1>(dz, in, B, g, cout, cin, splits, per, part, err, st);
 }
 
 cudaError_t sum_splits(const SumJobs &jobs, int count, cudaStream_t st) {
@@ -707,8 +707,9 @@ cudaError_t loss_final(const double *part, int n, const int *flag, double *out, 
 }
 
 cudaError_t adam(const NetParams &p, int layers, float lr, float b1, float b2, float eps, float c1,
-                 float c2, const int *flag, cudaStream_t st) {
-    k_adam<<<dim3(592, unsigned(layers)), 256, 0, st>>>(p, lr, b1, b2, eps, c1, c2, flag);
+                 float c2, long long step, const int *flag, long long *applied, cudaStream_t st) {
+    k_adam<<<dim3(592, unsigned(layers)), 256, 0, st>>>(p, lr, b1, b2, eps, c1, c2, step, flag,
+                                                        applied);
     return cudaGetLastError();
 }
 

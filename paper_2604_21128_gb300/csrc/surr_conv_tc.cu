@@ -35,7 +35,7 @@
 // separate pooling and upsampling, 53 32 41 47 47 90 131 113 93 71.
 //
 // Every wait on an mbarrier gives up after WAIT_NS of %globaltimer time; a CTA
-// that gives up raises conv_tc_error, lets its copies in flight land, frees
+// that gives up raises the caller's flag, lets its copies in flight land, frees
 // its TMEM and returns.  After such a timeout the launch's outputs are
 // undefined, and so is the TMEM it freed if the wait that ran out was on MMAs
 // still in flight (a genuine hang of the tensor pipe rather than a phase that
@@ -56,9 +56,9 @@ constexpr int EPI_WARPS = 8;                        // two per quarter of the TM
 constexpr int LOAD_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1;
 constexpr int CONV_THREADS = 32 * (EPI_WARPS + 2);
 
-__device__ int g_conv_tc_error;
-// Test hook (surr_test_stall_conv): CTA 0 of each launch waits for a phase
-// that never completes, so its bounded wait runs out.
+// Test hook (surr_test_stall_conv): CTA 0 of each launch, or (2) of each
+// EP_F32 launch, waits for a phase that never completes, so its bounded wait
+// runs out; launches that find their flag raised do not.
 __device__ int g_conv_tc_stall;
 
 // Shared-memory matrix descriptor (tcgen05 format): start address, leading
@@ -555,7 +555,9 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
-        if (ok && items > 0 && g_conv_tc_stall && blockIdx.x == 0)
+        if (ok && items > 0 && blockIdx.x == 0 && g_conv_tc_stall != 0 &&
+            (MODE == EP_F32 || g_conv_tc_stall == 1) &&
+            *static_cast<const volatile int *>(a.err) == 0)
             // the phase after the last one never completes
             ok = mbar_wait(&acc_full[(items - 1) & 1], (((items - 1) / 2) + 1) & 1, abort);
         if (!ok) abort_flag = 1;
@@ -563,7 +565,7 @@ k_conv3x3(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUte
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (tid == 0 && abort_flag) atomicExch(&g_conv_tc_error, 1);
+    if (tid == 0 && abort_flag) atomicExch(a.err, 1);
     if (warp == MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(pl.tcols)
@@ -758,19 +760,6 @@ cudaError_t conv3x3(const ConvArgs &a, ConvMode mode, cudaStream_t st) {
 
 cudaError_t conv_tc_stall(int on) {
     return cudaMemcpyToSymbol(g_conv_tc_stall, &on, sizeof(int));
-}
-
-cudaError_t conv_tc_error_ptr(int **dev) {
-    return cudaGetSymbolAddress(reinterpret_cast<void **>(dev), g_conv_tc_error);
-}
-
-cudaError_t conv_tc_error(int *flag, bool reset) {
-    cudaError_t e = cudaMemcpyFromSymbol(flag, g_conv_tc_error, sizeof(int));
-    if (e == cudaSuccess && reset) {
-        const int zero = 0;
-        e = cudaMemcpyToSymbol(g_conv_tc_error, &zero, sizeof(int));
-    }
-    return e;
 }
 
 }  // namespace surr

@@ -38,14 +38,12 @@ struct ConvArgs {
     bf16 *up;            // blocked, 2H x 2W, or null
     float *out_f;
     int n_out;
+    int *err;            // raised when one of the launch's mbarrier waits gives up
 };
 
 cudaError_t conv3x3(const ConvArgs &a, ConvMode mode, cudaStream_t st);
-// Reads (and with reset, clears) the flag a tcgen05 convolution sets when one
-// of its mbarrier waits gives up; its device address.
-cudaError_t conv_tc_error(int *flag, bool reset);
-cudaError_t conv_tc_error_ptr(int **dev);
-// Test hook: make one CTA of each convolution run out a wait.
+// Test hook: make one CTA run out a wait, in convolutions of every mode (1) or
+// of EP_F32 only (2), as long as the launch's flag is not raised.
 cudaError_t conv_tc_stall(int on);
 
 // A tensor map over a blocked BF16 tensor: box of bx pixels x by rows x bg
@@ -54,9 +52,9 @@ bool blocked_map(CUtensorMap *map, const bf16 *t, int B, int C, int H, int W, bo
                  int by, int bg);
 
 // part[split][co][tap][ci] = this split's sum over pixels of dz x shifted in
-// (both blocked; cout, cin 16 or multiples of 32).
+// (both blocked; cout, cin 16 or multiples of 32).  err: as in ConvArgs.
 cudaError_t weight_grad(const bf16 *dz, const bf16 *in, int B, int H, int W, int cout, int cin,
-                        int splits, float *part, cudaStream_t st);
+                        int splits, float *part, int *err, cudaStream_t st);
 // The network's splits for a level.
 int weight_grad_splits(int B, int H, int W);
 
@@ -91,14 +89,14 @@ cudaError_t pack_features(const float *f, int B, int H, int W, int feat, int cpa
 // part, dz (channel group 0 of `groups`) and its bias sums bpart[range][16].
 cudaError_t mse(const float *y, const float *t, int nout, int B, int H, int W, int groups, bf16 *dz,
                 double *part, float *bpart, cudaStream_t st);
-// out[0] = sum of part; out[1] = the convolutions' wait flag (0 or 1).
+// out[0] = sum of part; out[1] = the wait flag (0 or 1).
 cudaError_t loss_final(const double *part, int n, const int *flag, double *out, cudaStream_t st);
 
 // Adam on FP32 master weights [cout][tap][cin] and biases of all layers, and
 // the two BF16 copies the convolutions read: wb [tap][cin/8][cout][8] and the
 // flipped transpose wt [tap][cout/8][cin][8] (wt[t][co][ci] = w[co][8-t][ci]).
-// Skips everything while *flag is raised.  Without Adam (refresh), only the
-// copies are written.
+// Skips everything while *flag is raised, else writes `step` to *applied.
+// Without Adam (refresh), only the copies are written.
 constexpr int MAX_LAYERS = 10;
 struct LayerParams {
     float *w, *gw, *mw, *vw, *b, *gb, *mb, *vb;
@@ -107,7 +105,7 @@ struct LayerParams {
 };
 struct NetParams { LayerParams l[MAX_LAYERS]; };
 cudaError_t adam(const NetParams &p, int layers, float lr, float b1, float b2, float eps, float c1,
-                 float c2, const int *flag, cudaStream_t st);
+                 float c2, long long step, const int *flag, long long *applied, cudaStream_t st);
 cudaError_t refresh_copies(const NetParams &p, int layers, cudaStream_t st);
 
 // NHWC BF16 <-> blocked, weights [cout][tap][cin] -> [tap][cin/8][cout][8].

@@ -78,8 +78,9 @@ struct surr_net {
     double *lout;                              // loss and wait flag
     double *lhost = nullptr;                   // the same, pinned
     cudaEvent_t ldone = nullptr;
-    int *flag = nullptr;                       // the convolutions' wait flag
-    long long step = 0;
+    int *flag;                                 // raised by a wait that ran out
+    long long *applied;                        // Adam steps made (device)
+    long long step = 0;                        // Adam steps enqueued and not known to be skipped
     std::string err;
 };
 
@@ -154,6 +155,8 @@ size_t carve_all(surr_net *n) {
     // the lattice checks of surr_advance use 768 doubles of it
     n->lpart = carve<double>(p, size_t(std::max(768, bias_blocks(B, H, W))));
     n->lout = carve<double>(p, 2);
+    n->flag = carve<int>(p, 1);
+    n->applied = carve<long long>(p, 1);
     return size_t(p - n->mem);
 }
 
@@ -192,6 +195,7 @@ qla_status forward(surr_net *n, int B, float *y) {
         a.up = i >= 4 && i < 8 ? n->U[l - 1] : nullptr;
         a.out_f = y;
         a.n_out = NOUT;
+        a.err = n->flag;
         NCUDA(n, conv3x3(a, i == 9 ? EP_OUT : EP_ACT, n->stream), "surrogate: conv");
     }
     return QLA_OK;
@@ -206,7 +210,7 @@ qla_status conv_backward(surr_net *n, int i, int B, const bf16 *dz, float *d_in,
     const LayerParams &l = n->prm.l[i];
     const int splits = weight_grad_splits(B, h, w);
     NCUDA(n, weight_grad(dz, conv_input(n, i), B, h, w, s.cout, s.cin, splits, n->part[i],
-                         n->stream),
+                         n->flag, n->stream),
           "surrogate: weight grad");
     jobs.j[njobs++] = {n->part[i], l.gw, splits, (long long)n->nw[i], false};
     jobs.j[njobs++] = {n->bpart[i], l.gb, bias_blocks(B, h, w), s.cout, false};
@@ -220,6 +224,7 @@ qla_status conv_backward(surr_net *n, int i, int B, const bf16 *dz, float *d_in,
         a.cout = s.cin;
         a.w = l.wt;
         a.out_f = d_in;
+        a.err = n->flag;
         NCUDA(n, conv3x3(a, EP_F32, n->stream), "surrogate: input grad");
     }
     return QLA_OK;
@@ -259,17 +264,28 @@ qla_status backward(surr_net *n, int B) {
     return QLA_OK;
 }
 
-// After a stream synchronisation: did a tcgen05 convolution give up one of
-// its bounded waits since the last check?  (Its CTAs then skipped their
-// epilogues, so the outputs are not to be trusted.)
+// A bounded wait of one of this network's kernels ran out (its CTA skipped
+// its outputs, so they are not to be trusted).  The flag is cleared once
+// nothing enqueued reads it any more; Adam steps that found it raised made no
+// update and do not count.
+qla_status wait_ran_out(surr_net *n) {
+    long long applied = 0;
+    NCUDA(n, cudaMemcpyAsync(&applied, n->applied, sizeof applied, cudaMemcpyDeviceToHost,
+                             n->stream), "surrogate: step count");
+    NCUDA(n, cudaMemsetAsync(n->flag, 0, sizeof(int), n->stream), "surrogate: wait flag");
+    NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
+    n->step = applied;
+    return nfail(n, QLA_ETIMEOUT,
+                 "surrogate: a tensor-core wait ran out; results of tensor-core launches "
+                 "are undefined until the network is rebuilt");
+}
+
 qla_status tc_waits_ok(surr_net *n) {
     int flag = 0;
-    NCUDA(n, conv_tc_error(&flag, true), "surrogate: wait flag");
-    if (flag)
-        return nfail(n, QLA_ETIMEOUT,
-                     "surrogate: a tensor-core wait ran out; results of tensor-core launches "
-                     "are undefined until the network is rebuilt");
-    return QLA_OK;
+    NCUDA(n, cudaMemcpyAsync(&flag, n->flag, sizeof flag, cudaMemcpyDeviceToHost, n->stream),
+          "surrogate: wait flag");
+    NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
+    return flag ? wait_ran_out(n) : QLA_OK;
 }
 
 // The loss of n->Y, its gradient into dz9, and loss and wait flag on their
@@ -289,12 +305,7 @@ qla_status loss_begin(surr_net *n, int B, const float *target) {
 qla_status loss_end(surr_net *n, double *out) {
     NCUDA(n, cudaEventSynchronize(n->ldone), "surrogate: sync");
     *out = n->lhost[0];
-    if (n->lhost[1] != 0.0) {
-        // the flag is cleared only once nothing of this call reads it any more
-        NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
-        return tc_waits_ok(n);
-    }
-    return QLA_OK;
+    return n->lhost[1] != 0.0 ? wait_ran_out(n) : QLA_OK;
 }
 
 qla_status pack(surr_net *n, const float *feat, int B) {
@@ -450,7 +461,8 @@ qla_status surr_create(surr_net **out, int height, int width, int max_batch,
     n->mem = static_cast<char *>(workspace);
     carve_all(n);
     // the output layer's dz keeps zeros in its padded channels
-    if (conv_tc_error_ptr(&n->flag) != cudaSuccess ||
+    if (cudaMemsetAsync(n->flag, 0, sizeof(int), n->stream) != cudaSuccess ||
+        cudaMemsetAsync(n->applied, 0, sizeof(long long), n->stream) != cudaSuccess ||
         cudaMallocHost(&n->lhost, 16) != cudaSuccess ||
         cudaEventCreateWithFlags(&n->ldone, cudaEventDisableTiming) != cudaSuccess ||
         cudaMemsetAsync(n->dz9, 0, blocked_elems(max_batch, CPAD, height, width) * 2,
@@ -505,6 +517,7 @@ long long surr_param_count(const surr_net *n) {
 // real channel counts; ky, kx = dy + 1, dx + 1.
 static qla_status params_io(surr_net *n, float *host, bool get, bool grads) {
     if (!n || !host) return QLA_EINVAL;
+    int flag = 0;   // read with the last layer
     size_t off = 0;
     for (int i = 0; i < NCONV; ++i) {
         const ConvSpec s = spec(i);
@@ -516,6 +529,9 @@ static qla_status params_io(surr_net *n, float *host, bool get, bool grads) {
                   "surrogate: params");
             NCUDA(n, cudaMemcpyAsync(b.data(), db, s.cout * 4, cudaMemcpyDeviceToHost, n->stream),
                   "surrogate: params");
+            if (get && i == NCONV - 1)
+                NCUDA(n, cudaMemcpyAsync(&flag, n->flag, sizeof flag, cudaMemcpyDeviceToHost,
+                                         n->stream), "surrogate: wait flag");
             NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
         }
         for (int co = 0; co < s.cout_real; ++co)
@@ -542,7 +558,7 @@ static qla_status params_io(surr_net *n, float *host, bool get, bool grads) {
         NCUDA(n, refresh_copies(n->prm, NCONV, n->stream), "surrogate: params");
         NCUDA(n, cudaStreamSynchronize(n->stream), "surrogate: sync");
     }
-    return QLA_OK;
+    return flag ? wait_ran_out(n) : QLA_OK;
 }
 
 qla_status surr_get_params(surr_net *n, float *host) { return params_io(n, host, true, false); }
@@ -571,21 +587,23 @@ qla_status surr_loss_grad(surr_net *n, const float *feat_dev, const float *targe
 }
 
 // The whole step is enqueued before the host waits for the loss, so the GPU
-// does not idle between the loss and the backward pass; Adam skips its update
-// if a convolution's wait ran out.
+// does not idle between the loss and the backward pass.  If a wait ran out,
+// Adam skips its update: a wait before the loss is reported here, one after
+// it by the next call that reads the flag, which takes the step back.
 qla_status surr_train_step(surr_net *n, const float *feat_dev, const float *target_dev, int B,
                            float lr, double *loss_out) {
     if (!n || !feat_dev || !target_dev) return QLA_EINVAL;
     qla_status s = enqueue_grad(n, feat_dev, target_dev, B);
     if (s != QLA_OK) return s;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const double step = double(n->step + 1);
-    const float c1 = float(1.0 - std::pow(0.9, step));
-    const float c2 = float(1.0 - std::pow(0.999, step));
-    NCUDA(n, adam(n->prm, NCONV, lr, b1, b2, eps, c1, c2, n->flag, n->stream), "surrogate: adam");
+    const long long step = n->step + 1;
+    const float c1 = float(1.0 - std::pow(0.9, double(step)));
+    const float c2 = float(1.0 - std::pow(0.999, double(step)));
+    NCUDA(n, adam(n->prm, NCONV, lr, b1, b2, eps, c1, c2, step, n->flag, n->applied, n->stream),
+          "surrogate: adam");
     double l = 0.0;
     if ((s = loss_end(n, &l)) != QLA_OK) return s;
-    n->step++;
+    n->step = step;
     if (loss_out) *loss_out = l;
     return QLA_OK;
 }
@@ -674,6 +692,15 @@ struct Scratch {
                                                                      : nullptr;
     }
 };
+
+// Waits for the stream; QLA_ETIMEOUT if a wait of the call's kernels ran out.
+qla_status raw_waits_ok(const int *flag_dev, cudaStream_t st) {
+    int flag = 0;
+    if (cudaMemcpyAsync(&flag, flag_dev, sizeof flag, cudaMemcpyDeviceToHost, st) ||
+        cudaStreamSynchronize(st))
+        return QLA_ECUDA;
+    return flag ? QLA_ETIMEOUT : QLA_OK;
+}
 }  // namespace
 
 extern "C" qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W, int cin,
@@ -682,11 +709,12 @@ extern "C" qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W,
     if (!in_bf16 || !w_bf16 || !out_f32 || B < 1 || H < 1 || W < 1 || cin % 32 || cout % 32)
         return QLA_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    Scratch sx(st), sw(st), so(st);
+    Scratch sx(st), sw(st), so(st), sf(st);
     bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));
     bf16 *w = sw.get<bf16>(size_t(cout) * 9 * cin);
     float *o = so.get<float>(size_t(B) * H * W * cout);
-    if (!x || !w || !o) {
+    int *flag_dev = sf.get<int>(1);
+    if (!x || !w || !o || !flag_dev || cudaMemsetAsync(flag_dev, 0, sizeof(int), st)) {
         cudaGetLastError();
         return QLA_ECUDA;
     }
@@ -699,19 +727,17 @@ extern "C" qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W,
     a.cout = cout;
     a.w = w;
     a.out_f = o;
+    a.err = flag_dev;
     if (nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) != cudaSuccess ||
         block_weights(static_cast<const bf16 *>(w_bf16), cout, cin, w, st) != cudaSuccess ||
         conv3x3(a, EP_F32, st) != cudaSuccess ||
         blocked_to_nhwc_f32(o, B, H, W, cout, out_f32, st) != cudaSuccess)
         return QLA_ECUDA;
-    int flag = 0;
-    if (cudaStreamSynchronize(st) != cudaSuccess || conv_tc_error(&flag, true) != cudaSuccess)
-        return QLA_ECUDA;
-    return flag ? QLA_ETIMEOUT : QLA_OK;
+    return raw_waits_ok(flag_dev, st);
 }
 
 extern "C" qla_status surr_test_stall_conv(int on) {
-    return conv_tc_stall(on ? 1 : 0) == cudaSuccess ? QLA_OK : QLA_ECUDA;
+    return conv_tc_stall(on == 2 ? 2 : on ? 1 : 0) == cudaSuccess ? QLA_OK : QLA_ECUDA;
 }
 
 extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_bf16, int B, int H,
@@ -720,20 +746,24 @@ extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_b
     if (!dz_bf16 || !in_bf16 || !part || !dw_f32 || cin % 32 || cout % 32 || splits < 1)
         return QLA_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    Scratch sz(st), sx(st);
+    Scratch sz(st), sx(st), sf(st);
     bf16 *z = sz.get<bf16>(blocked_elems(B, cout, H, W));
     bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));
-    if (!z || !x) {
+    int *flag_dev = sf.get<int>(1);
+    if (!z || !x || !flag_dev || cudaMemsetAsync(flag_dev, 0, sizeof(int), st)) {
         cudaGetLastError();
         return QLA_ECUDA;
     }
     SumJobs jobs{};
     jobs.j[0] = {part, dw_f32, splits, (long long)cout * 9 * cin, false};
-    return nhwc_to_blocked(static_cast<const bf16 *>(dz_bf16), B, H, W, cout, z, st) ==
-                       cudaSuccess &&
-                   nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) ==
-                       cudaSuccess &&
-                   weight_grad(z, x, B, H, W, cout, cin, splits, part, st) == cudaSuccess &&
-                   sum_splits(jobs, 1, st) == cudaSuccess
-               ? QLA_OK : QLA_ECUDA;
+    if (nhwc_to_blocked(static_cast<const bf16 *>(dz_bf16), B, H, W, cout, z, st) != cudaSuccess ||
+        nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) != cudaSuccess ||
+        weight_grad(z, x, B, H, W, cout, cin, splits, part, flag_dev, st) != cudaSuccess ||
+        sum_splits(jobs, 1, st) != cudaSuccess)
+        return QLA_ECUDA;
+    // a stream that is being captured cannot be waited for
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+        return QLA_OK;
+    return raw_waits_ok(flag_dev, st);
 }

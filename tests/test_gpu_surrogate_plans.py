@@ -1,6 +1,7 @@
-"""Convolution layouts that the small images of test_gpu_surrogate.py do not
-reach: wide output slices, streamed weights, several tiles per block, against
-FP64 sums on BF16 data."""
+"""The surrogate's convolutions beyond the small images of
+test_gpu_surrogate.py: wide output slices, streamed weights and several tiles
+per block against FP64 sums on BF16 data, and what its calls report when a
+device wait runs out."""
 import ctypes
 
 import numpy as np
@@ -51,3 +52,55 @@ def test_wide_inputs_are_taken(B, H, W, cin, cout):
     # products of BF16 values are exact; the FP32 accumulation of 9 cin terms
     # rounds (~sqrt(9 cin) 6e-8 relative)
     assert float(torch.linalg.norm(out - want) / torch.linalg.norm(want)) <= 1e-5
+
+
+def small_net(seed=3):
+    import torch
+    from paper_2604_21128_gb300 import surrogate
+    net = surrogate.Surrogate(32, 48, max_batch=2, seed=seed)
+    rng = np.random.default_rng(seed)
+    x = torch.tensor(rng.standard_normal((2, 32, 48, 6)), dtype=torch.float32, device="cuda")
+    t = torch.tensor(rng.standard_normal((2, 32, 48, 3)) * 0.1, dtype=torch.float32, device="cuda")
+    return net, x, t
+
+
+def test_wait_that_runs_out_in_the_backward_pass_is_reported():
+    """The loss is out before the backward pass: a wait that runs out there
+    leaves the parameters alone, is reported when they are read, does not
+    count as a step and does not touch another network."""
+    lib = qla.load()
+    net, x, t = small_net()
+    other, _, _ = small_net()
+    want, _, _ = small_net()
+    for n in (net, want):
+        n.train_step(x, t, 1e-3)
+    before = net.params()
+    assert lib.surr_test_stall_conv(2) == 0        # input gradients only
+    try:
+        loss = net.train_step(x, t, 1e-3)
+        other_before = other.params()              # no timeout of its own
+        with pytest.raises(qla.QLAError) as e:
+            net.params()
+    finally:
+        assert lib.surr_test_stall_conv(0) == 0
+    assert e.value.status == 5                     # QLA_ETIMEOUT
+    assert np.array_equal(net.params(), before)
+    # the next step is the second again
+    assert net.train_step(x, t, 1e-3) == loss == want.train_step(x, t, 1e-3)
+    assert np.array_equal(net.params(), want.params())
+    assert np.array_equal(other.params(), other_before)
+
+
+def test_gradient_with_a_wait_that_ran_out_is_refused():
+    lib = qla.load()
+    net, x, t = small_net()
+    want = net.loss_grad(x, t)
+    assert lib.surr_test_stall_conv(2) == 0
+    try:
+        with pytest.raises(qla.QLAError) as e:
+            net.loss_grad(x, t)
+    finally:
+        assert lib.surr_test_stall_conv(0) == 0
+    assert e.value.status == 5                     # QLA_ETIMEOUT
+    got = net.loss_grad(x, t)
+    assert got[0] == want[0] and np.array_equal(got[1], want[1])

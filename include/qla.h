@@ -301,7 +301,9 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * after about two seconds of SM cycles; the next synchronising read
  * (qla_energy, qla_energy_box, qla_divergence, qla_probe, qla_fields,
  * qla_get_state) then returns QLA_ETIMEOUT and the state is undefined until
- * it is set again (steps launched before that read do no work).
+ * it is set again (steps launched before that read do no work).  Once such a
+ * launch has gone into a stream capture, every such read looks at the flag,
+ * so the one after a replay reports that replay's wait.
  * QLA_KERNEL_MARCH_STEP = the plateau split, one launch per step;
  * QLA_KERNEL_MARCH_FLOW = dataflow steps on every lattice the plateau
  * split takes (32-row segments unless qla_set_march_tuning sets rows). */

@@ -21,9 +21,16 @@ static bool march_ok(const qla_ctx *c) {
     return march_supported(c) && offsets32_ok(size_t(c->P), c->plane_elems);
 }
 
-cudaError_t reset_wait_flag(qla_ctx *c) {
-    return c->flow_unchecked ? cudaSuccess
-                             : cudaMemsetAsync(c->wait_flag, 0, sizeof(int), c->stream);
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();   // the legacy stream while another thread captures
+    return true;
+}
+
+void note_waits(qla_ctx *c) {
+    c->flow_unchecked = true;
+    c->flow_captured = c->flow_captured || capturing(c->stream);
 }
 
 Layout layout_for(int nx, int ny, int prec, unsigned flags) {
@@ -125,11 +132,11 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-// After a synchronisation of the context's stream: QLA_ETIMEOUT if a
-// step launched since the last check gave up a wait.  flag: the wait flag
-// where the call has already copied it, else null.
+// After a synchronisation of the context's stream: QLA_ETIMEOUT, and the wait
+// flag cleared, if a step since the last check gave up a wait.  flag: the wait
+// flag where the call has already copied it, else null.
 qla_status check_flow(qla_ctx *c, const char *what, const int *flag = nullptr) {
-    if (!c->flow_unchecked) return QLA_OK;
+    if (!c->flow_unchecked && !c->flow_captured) return QLA_OK;
     int v = 0;
     if (flag) {
         v = *flag;
@@ -138,10 +145,25 @@ qla_status check_flow(qla_ctx *c, const char *what, const int *flag = nullptr) {
         if (e != cudaSuccess) return cuda_fail(c, e, what);
     }
     c->flow_unchecked = false;
-    if (v)
+    if (v) {
+        cudaError_t e = cudaMemsetAsync(c->wait_flag, 0, sizeof(int), c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, what);
         return fail(c, QLA_ETIMEOUT,
                     "%s: a step's wait for its neighbours ran out; the state is undefined "
                     "until it is set again", what);
+    }
+    return QLA_OK;
+}
+
+// A new state has been enqueued: no potential step is pending, and a wait that
+// ran out before it concerned the old state.
+qla_status new_state(qla_ctx *c, const char *what) {
+    if (c->flow_unchecked || c->flow_captured)
+        QLA_CUDA(c, cudaMemsetAsync(c->wait_flag, 0, sizeof(int), c->stream), what);
+    c->flow_unchecked = false;
+    c->has_state = true;
+    c->pending_v = false;
     return QLA_OK;
 }
 
@@ -259,8 +281,9 @@ qla_status qla_init_grid(qla_ctx **out, int nx, int ny, double delta, int precis
         c->items = reinterpret_cast<int *>(c->ws + L.items);
         c->items_cap = L.items_cap;
     }
-    // both state buffers start at zero (pad columns included)
-    if (cudaMemsetAsync(c->ws + L.state[0], 0, L.midx - L.state[0], c->stream) != cudaSuccess) {
+    // both state buffers start at zero (pad columns included), the wait flag too
+    if (cudaMemsetAsync(c->ws + L.state[0], 0, L.midx - L.state[0], c->stream) != cudaSuccess ||
+        cudaMemsetAsync(c->wait_flag, 0, sizeof(int), c->stream) != cudaSuccess) {
         cudaGetLastError();
         if (c->owns_ws) cudaFree(c->ws);
         delete c;
@@ -356,10 +379,7 @@ qla_status qla_set_packet(qla_ctx *c, const qla_packet *p) {
                                     c->plane_elems * (c->prec == QLA_FP64 ? 8 : 4) * 6, c->stream),
                  "qla_set_packet: clear");
     QLA_CUDA(c, launch_packet(c, *p), "qla_set_packet: kernel");
-    c->has_state = true;
-    c->pending_v = false;
-    c->flow_unchecked = false;
-    return QLA_OK;
+    return new_state(c, "qla_set_packet: wait flag");
 }
 
 qla_status qla_set_packet_window(qla_ctx *c, const qla_packet *p, int i0, int j0, int gnx,
@@ -386,10 +406,7 @@ qla_status qla_set_packet_window(qla_ctx *c, const qla_packet *p, int i0, int j0
                                     c->plane_elems * (c->prec == QLA_FP64 ? 8 : 4) * 6, c->stream),
                  "qla_set_packet_window: clear");
     QLA_CUDA(c, launch_packet_window(c, *p, i0, j0, gnx, gny), "qla_set_packet_window: kernel");
-    c->has_state = true;
-    c->pending_v = false;
-    c->flow_unchecked = false;
-    return QLA_OK;
+    return new_state(c, "qla_set_packet_window: wait flag");
 }
 
 size_t qla_box_bytes(const qla_ctx *c, int w, int h) {
@@ -473,10 +490,7 @@ qla_status qla_set_state(qla_ctx *c, const double *q_host) {
     // the staging plane is reused per component: wait before the host buffer
     // may change and before the next copy overwrites staging
     QLA_CUDA(c, cudaStreamSynchronize(c->stream), "qla_set_state: sync");
-    c->has_state = true;
-    c->pending_v = false;
-    c->flow_unchecked = false;   // a wait that ran out concerned the old state
-    return QLA_OK;
+    return new_state(c, "qla_set_state: wait flag");
 }
 
 qla_status qla_get_state(qla_ctx *c, double *q_host) {

@@ -402,14 +402,18 @@ struct qla_ctx {
         size_t off_xdep = 0, off_ydep = 0, off_ctr = 0;
     } uplan;
     // device flag that a wait between tiles or units of steps raises when it
-    // runs out (behind the reduction results, so one copy brings both), and
-    // the resident tile steps' counters
+    // runs out (behind the reduction results, so one copy brings both; it
+    // stays raised until a read reports it or the state is set, and launches
+    // that find it raised give up their waits), and the resident tile steps'
+    // counters
     int *wait_flag = nullptr;
     unsigned *tile_done = nullptr;
     // launches that wait on one another's tiles or units: one whose wait flag
-    // has not been read yet, each wait's limit in SM cycles, and a test hook
-    // (the handed-out unit index whose completion is withheld, -1 none)
-    bool flow_unchecked = false;
+    // has not been read yet, one that went into a stream capture (replays of
+    // which the host does not see: every read then looks at the flag), each
+    // wait's limit in SM cycles, and a test hook (the handed-out unit index
+    // whose completion is withheld, -1 none)
+    bool flow_unchecked = false, flow_captured = false;
     long long flow_budget = 1LL << 32;
     long long flow_withhold = -1;
     qla_status sticky = QLA_OK;
@@ -495,8 +499,11 @@ cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done
 bool tile_steps_pay(const qla_ctx *c);
 // An FP64 marching step's time in item rows (see pick_segment64).
 double march64_rows(const qla_ctx *c);
-// Clears the wait flag unless launches since its last read may have raised it.
-cudaError_t reset_wait_flag(qla_ctx *c);
+// Whether the stream is being captured, or cannot be asked now.
+bool capturing(cudaStream_t st);
+// Notes a launch with waits on the context's stream: the next synchronising
+// read looks at the wait flag, every later one if the stream is being captured.
+void note_waits(qla_ctx *c);
 bool march_supported(const qla_ctx *c);
 int march_lane_cols(const qla_ctx *c);
 }  // namespace qla

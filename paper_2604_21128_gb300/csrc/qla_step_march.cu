@@ -514,10 +514,6 @@ cudaError_t launch_flow(qla_ctx *c, const void *in, void *out, long long n_steps
     char *base = reinterpret_cast<char *>(c->items);
     unsigned *ctr = reinterpret_cast<unsigned *>(base + u.off_ctr);
     int *err = c->wait_flag;
-    {
-        const cudaError_t e = reset_wait_flag(c);
-        if (e != cudaSuccess) return e;
-    }
     // units x steps of one launch below 2^31, item counters below 2^32
     const long long per = std::max(1LL, std::min<long long>((1LL << 31) / u.n_list, 1LL << 26));
     float *a = static_cast<float *>(const_cast<void *>(in)), *b = static_cast<float *>(out);
@@ -534,7 +530,7 @@ cudaError_t launch_flow(qla_ctx *c, const void *in, void *out, long long n_steps
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         c->launches++;
-        c->flow_unchecked = true;
+        note_waits(c);
         if (k & 1) std::swap(a, b);
         left -= k;
     }

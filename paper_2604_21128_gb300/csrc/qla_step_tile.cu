@@ -416,9 +416,7 @@ cudaError_t launch_tile_t(qla_ctx *c, const void *in, void *out, bool vin, long 
             nullptr, nullptr, 0, -1);
         return cudaGetLastError();
     }
-    cudaError_t e = reset_wait_flag(c);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(c->tile_done, 0, size_t(tg.n_tx) * tg.n_ty * 4, c->stream);
+    cudaError_t e = cudaMemsetAsync(c->tile_done, 0, size_t(tg.n_tx) * tg.n_ty * 4, c->stream);
     if (e != cudaSuccess) return e;
     int steps = int(n_steps);
     int *err = c->wait_flag;
@@ -427,9 +425,8 @@ cudaError_t launch_tile_t(qla_ctx *c, const void *in, void *out, bool vin, long 
                     &c->plane_elems, &tg, &vin, &steps, &c->tile_done, &err, &budget, &withhold};
     e = cudaLaunchCooperativeKernel(kern, dim3(unsigned(tg.n_tx * tg.n_ty)), dim3(32 * warps),
                                     args, K::SMEM, c->stream);
-    if (e != cudaSuccess) return e;
-    c->flow_unchecked = true;
-    return cudaSuccess;
+    if (e == cudaSuccess) note_waits(c);
+    return e;
 }
 
 template <typename T>

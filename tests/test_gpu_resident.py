@@ -79,3 +79,46 @@ def test_tile_wait_runs_out_without_fault():
         g.step(6)
         out.append(g.get_state())
     assert np.array_equal(out[0], out[1])
+
+
+def test_captured_steps_report_their_waits():
+    """Steps captured into graphs: a replay whose wait runs out is reported by
+    the read after it, each time; another graph of the same context, captured
+    before any read, then runs as it should."""
+    import torch
+    nx, ny = 96, 72
+    n = inputs.random_medium(nx, ny, seed=3)
+    q0 = inputs.random_state(nx, ny, seed=4)
+    stream = torch.cuda.Stream()
+    with qla.Grid(nx, ny, 1.0, "fp64", stream=stream) as g:
+        def start():
+            g.set_state(q0)
+            g.step(2)
+        g.set_medium(n)
+        start()
+        graphs = []
+        for withhold in (3, -1):
+            g.debug_flow(budget_cycles=2_000_000 if withhold >= 0 else 0, withhold_unit=withhold)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                g.step(6)
+            graphs.append(graph)
+        g.energy()
+        for _ in range(2):
+            with torch.cuda.stream(stream):
+                graphs[0].replay()
+            with pytest.raises(qla.QLAError) as e:
+                g.energy()
+            assert e.value.status == 5     # QLA_ETIMEOUT
+            start()
+        g.energy()
+        with torch.cuda.stream(stream):
+            graphs[1].replay()
+        got = g.get_state()
+        del graphs
+    with qla.Grid(nx, ny, 1.0, "fp64") as g:
+        g.set_step_kernel("tile")
+        g.set_medium(n)
+        g.set_state(q0)
+        g.step(8)
+        assert np.array_equal(got, g.get_state())

@@ -282,8 +282,8 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * as one tile per SM goes, double-single contexts excepted): a qla_step call
  * runs all its steps in one cooperative launch of the tile kernel, every
  * tile waiting for its eight neighbours between steps; the results are those
- * of one launch per step bit for bit.  Lattices the plateau split takes, of
- * 2^18 sites or more, keep the split for calls of one to three steps.
+ * of one launch per step bit for bit.  A context with a tuning set
+ * (qla_set_march_tuning) takes the marching kernel instead.
  * QLA_KERNEL_TILE = the tile kernel, one launch per step.
  * QLA_KERNEL_MARCH_PLAIN = the marching kernel without the split.
  * Dataflow steps (plateau split, lattices with at least about three work
@@ -396,7 +396,9 @@ qla_status qla_energy_noalloc(const void *planes, int precision, int n_planes, i
  * chains per warp), 2 or 4 = that many adjacent columns per lane (scalar
  * FP32; 2 is the default).  Other contexts always use 2.  rows = rows per work
  * item (0 = chosen from the occupancy so one wave of items fills the GPU;
- * else rounded up to a multiple of 4).  Results do not depend on either.
+ * else rounded up to a multiple of 4).  A value other than 0 of either makes
+ * QLA_KERNEL_AUTO take the marching kernel on every lattice it supports.
+ * Results do not depend on either.
  * QLA_EINVAL for other values. */
 qla_status qla_set_march_tuning(qla_ctx *ctx, int lane_cols, int rows);
 
@@ -671,10 +673,12 @@ long long qla_launch_count(const qla_ctx *ctx);
 /* The plateau plan of the FP32 E_z marching step (see qla_set_step_kernel),
  * as built for the current medium and tuning by the last marching step:
  * work items (128-column windows x row segments) per step, items run on the
- * plateau path, and distinct plateau records among them.  All zero when no
- * plan is in use (other contexts, another kernel, no plateau item, or no
- * step since the medium or the tuning changed).  Any output pointer may be
- * NULL.  QLA_EINVAL for a null ctx. */
+ * plateau path, and distinct plateau records among them.  For a lattice whose
+ * steps ran on resident tiles instead, the plan of the marching step they
+ * take the place of, built by this call (which then synchronises the
+ * context's stream).  All zero when no plan is in use (other contexts,
+ * another kernel, no plateau item, or no step since the medium or the tuning
+ * changed).  Any output pointer may be NULL.  QLA_EINVAL for a null ctx. */
 qla_status qla_march_plan(const qla_ctx *ctx, int *n_items, int *n_plateau_items, int *n_sets);
 
 /* Text of the last error on this context ("" if none); valid until the next

@@ -527,7 +527,9 @@ qla_status qla_step(qla_ctx *c, long long n_steps) {
     // V applied by the step that computes it (tensor media, the LCU branches)
     // rather than by the next one
     const bool v_now = (c->tensor && c->P == 6) || c->vmode == V_LCU;
-    if (c->step_kernel == QLA_KERNEL_AUTO && !c->dstable) {
+    // a tuning asks for the marching kernel wherever it runs
+    const bool tuned = (c->march_lx != 0 || c->march_seg != 0) && march_ok(c);
+    if (c->step_kernel == QLA_KERNEL_AUTO && !c->dstable && !tuned) {
         // small lattices: every tile resident, many steps per launch
         for (long long k = 0; n_steps > 0; n_steps -= k) {
             QLA_CUDA(c, launch_steps_resident(c, n_steps, &k), "qla_step: resident tiles");
@@ -568,7 +570,8 @@ qla_status qla_step(qla_ctx *c, long long n_steps) {
                        c->step_kernel == QLA_KERNEL_MARCH_PLAIN ||
                        c->step_kernel == QLA_KERNEL_MARCH_STEP ||
                        c->step_kernel == QLA_KERNEL_MARCH_FLOW ||
-                       (c->step_kernel == QLA_KERNEL_AUTO && march_ok(c) && !tile_steps_pay(c));
+                       (c->step_kernel == QLA_KERNEL_AUTO &&
+                        (tuned || (march_ok(c) && !tile_steps_pay(c))));
     if (march) {
         // all n steps in persistent dataflow launches where the context
         // takes them
@@ -763,9 +766,18 @@ qla_status qla_debug_flow(qla_ctx *c, long long budget_cycles, long long withhol
     return QLA_OK;
 }
 
-qla_status qla_march_plan(const qla_ctx *c, int *n_items, int *n_plateau_items, int *n_sets) {
-    if (!c) return QLA_EINVAL;
+qla_status qla_march_plan(const qla_ctx *cc, int *n_items, int *n_plateau_items, int *n_sets) {
+    if (!cc) return QLA_EINVAL;
+    // the plan is scratch of the context that a query may fill in (contexts
+    // are never const objects: qla_init_grid makes them)
+    qla_ctx *c = const_cast<qla_ctx *>(cc);
     const auto &u = c->uplan;
+    if (c->sticky == QLA_OK && c->plan_due == c->medium_gen && u.gen != c->medium_gen &&
+        march_ok(c) && !capturing(c->stream)) {
+        DeviceGuard dg(c->device);
+        if (!dg.ok) return fail(c, QLA_ECUDA, "qla_march_plan: cannot select device");
+        QLA_CUDA(c, build_march_plan(c), "qla_march_plan: plan");
+    }
     const bool live = u.gen == c->medium_gen && u.n_uniform > 0;
     if (n_items) *n_items = live ? u.n_items : 0;
     if (n_plateau_items) *n_plateau_items = live ? u.n_uniform : 0;

@@ -401,6 +401,9 @@ struct qla_ctx {
         int n_wx = 0, shift = 0;
         size_t off_xdep = 0, off_ydep = 0, off_ctr = 0;
     } uplan;
+    // the medium that resident tile steps ran on last: qla_march_plan builds
+    // the plan of the marching steps that they take the place of
+    long long plan_due = -1;
     // device flag that a wait between tiles or units of steps raises when it
     // runs out (behind the reduction results, so one copy brings both; it
     // stays raised until a read reports it or the state is set, and launches
@@ -493,6 +496,7 @@ cudaError_t launch_step_flow(qla_ctx *c, long long n_steps, bool *done);
 // The steps of a lattice whose tiles are all resident at once, in one launch
 // from c->state[c->cur] with c->pending_v; *done steps were enqueued (0 where
 // the lattice has too many tiles), the result in state[c->cur ^ (*done & 1)].
+// (For contexts without a marching tuning, see qla_step.)
 cudaError_t launch_steps_resident(qla_ctx *c, long long n_steps, long long *done);
 // Whether an automatic context's steps go to the tile kernel although the
 // marching kernel takes its lattice.
@@ -504,6 +508,9 @@ bool capturing(cudaStream_t st);
 // Notes a launch with waits on the context's stream: the next synchronising
 // read looks at the wait flag, every later one if the stream is being captured.
 void note_waits(qla_ctx *c);
+// Builds the plateau plan that marching steps of the context take, if it
+// splits by plateaus; synchronises its stream.
+cudaError_t build_march_plan(qla_ctx *c);
 bool march_supported(const qla_ctx *c);
 int march_lane_cols(const qla_ctx *c);
 }  // namespace qla

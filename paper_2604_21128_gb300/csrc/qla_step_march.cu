@@ -606,6 +606,7 @@ int split6_segment(const qla_ctx *c) {
     return best;
 }
 
+// Without buffers (out null) only the plan of the E_z plateau split is built.
 template <typename T, int P, int LX, int VM, bool VIN>
 cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
     using V = Variant<T, P, LX, VM, VIN>;
@@ -661,10 +662,12 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
                 const cudaError_t e = ensure_plateau_plan(c, pseg, fseg > 0);
                 if (e != cudaSuccess) return e;
             }
+            if (!out) return cudaSuccess;
             if (u.gen == c->medium_gen && u.seg == pseg && u.n_uniform > 0)
                 return launch_split<VM, VIN>(c, in, out);
         }
     }
+    if (!out) return cudaSuccess;
     if constexpr (std::is_same<T, float>::value && P == 6) {
         if (c->items && c->step_kernel != QLA_KERNEL_MARCH_PLAIN && c->nx % 4 == 0 &&
             c->nx >= PW) {
@@ -788,6 +791,12 @@ cudaError_t launch_step_march(qla_ctx *c, const void *in, void *out, bool vin) {
     case 4: return launch_vm<float, 3, 4>(c, in, out, vin);
     default: return launch_vm<float, 3, 2>(c, in, out, vin);
     }
+}
+
+cudaError_t build_march_plan(qla_ctx *c) {
+    if (c->prec != QLA_FP32 || c->P != 3 || march_lane_cols(c) != 2 || !march_supported(c))
+        return cudaSuccess;
+    return launch_vm<float, 3, 2>(c, nullptr, nullptr, c->pending_v);
 }
 
 double march64_rows(const qla_ctx *c) {

@@ -122,3 +122,57 @@ def test_captured_steps_report_their_waits():
         g.set_state(q0)
         g.step(8)
         assert np.array_equal(got, g.get_state())
+
+
+@pytest.mark.parametrize("calls", [(1, 2, 3), (8,)])
+def test_short_calls_take_resident_tiles_and_a_plan_is_described(calls):
+    """512^2 E_z lattices: calls of any length are one launch each, and the plan
+    of the marching step is described when asked for."""
+    nx = ny = 512
+    n = np.full((ny, nx), 2.0)
+    n[:, : nx // 3] = 1.0
+    q0 = inputs.random_state(nx, ny, seed=9, planes=3)
+    out = {}
+    for kernel in ("auto", "tile", "march"):
+        with qla.Grid(nx, ny, 1.0, "fp32", te_only=True) as g:
+            g.set_step_kernel(kernel)
+            g.set_medium(n)
+            g.set_state(q0)
+            assert g.march_plan == (0, 0, 0)       # no step yet
+            before = g.launches
+            for k in calls:
+                g.step(k)
+            out[kernel] = g.launches - before, g.get_state(), g.march_plan
+            g.set_medium(n)
+            assert g.march_plan == (0, 0, 0)
+    assert out["auto"][0] == len(calls) and out["tile"][0] == sum(calls)
+    assert np.array_equal(out["auto"][1], out["tile"][1])
+    assert np.array_equal(out["auto"][1], out["march"][1])
+    assert out["auto"][2] == out["march"][2] and out["auto"][2][1] > 0
+    assert out["tile"][2] == (0, 0, 0)
+
+
+@pytest.mark.parametrize("precision,te,lane_cols,rows",
+                         [("fp32", True, 1, 0), ("fp32", True, 0, 32), ("fp64", True, 0, 16),
+                          ("fp32", False, 0, 8)])
+def test_a_tuning_takes_the_marching_kernel(precision, te, lane_cols, rows):
+    nx, ny = 128, 96
+    n = inputs.random_medium(nx, ny, seed=5, lo=1.0, hi=2.5)
+    q0 = inputs.random_state(nx, ny, seed=6, planes=3 if te else 6)
+    out = {}
+    for kernel in ("auto", "march_step" if precision == "fp32" and te else "march"):
+        with qla.Grid(nx, ny, 1.0, precision, te_only=te) as g:
+            g.set_step_kernel(kernel)
+            g.set_march_tuning(lane_cols, rows)
+            g.set_medium(n)
+            g.set_state(q0)
+            before = g.launches
+            g.step(7)
+            out[kernel] = g.launches - before, g.get_state()
+            g.set_march_tuning()                   # resident tiles again
+            before = g.launches
+            g.step(5)
+            if kernel == "auto":
+                assert g.launches - before == 1
+    (a, sa), (b, sb) = out.values()
+    assert a == b == 7 and np.array_equal(sa, sb)

@@ -399,12 +399,12 @@ qla_status build_units(qla_batch *b, int rows, int *n_units, std::vector<BatchIn
     std::vector<long long> gens(b->count);
     for (int k = 0; k < b->count; ++k) gens[k] = b->inst[k]->medium_gen;
     const bool keep = b->list_units > 0 && b->list_rows == rows && b->list_gens == gens;
+    const int height = rows > 0 ? rows : auto_rows(b, PWOUT, 128);
     std::vector<int> segs(b->count), nwx(b->count), nitems(b->count);
     std::vector<size_t> at(b->count + 1, 0);
     for (int k = 0; k < b->count; ++k) {
         qla_ctx *c = b->inst[k];
-        int seg = rows > 0 ? rows : auto_rows(b, PWOUT, 128);
-        seg = (seg + 3) / 4 * 4;
+        int seg = (height + 3) / 4 * 4;
         if (seg > c->ny) seg = (c->ny + 3) / 4 * 4;
         segs[k] = seg;
         nwx[k] = (c->nx + PWOUT - 1) / PWOUT;
@@ -481,13 +481,13 @@ qla_status build_items(qla_batch *b, int lx, int rows, int *n_items,
                        std::vector<BatchInst> &hinst) {
     if (kernels(b, lx).plateau) return build_units(b, rows, n_items, hinst);
     const int wout = window_out(lx);
+    const int height = rows > 0 ? rows : auto_rows(b, wout, 256);
     b->list_units = 0;   // the items replace a unit list
     std::vector<BatchItem> items;
     hinst.resize(b->count);
     for (int k = 0; k < b->count; ++k) {
         qla_ctx *c = b->inst[k];
-        int seg = rows > 0 ? rows : auto_rows(b, wout, 256);
-        seg = (seg + 3) / 4 * 4;
+        int seg = (height + 3) / 4 * 4;
         if (seg > c->ny) seg = (c->ny + 3) / 4 * 4;
         const int n_wx = (c->nx + wout - 1) / wout, n_wy = (c->ny + seg - 1) / seg;
         BatchInst &I = hinst[k];

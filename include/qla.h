@@ -268,8 +268,11 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * lattice, including one whose live planes exceed its 32-bit element
  * offsets: planes x ny x padded nx > 2^32).  Both compute the same operator sequence; FP64 results agree to
  * rounding order.
- * Plateau split (FP32 E_z contexts, two columns per lane, nx a multiple of
- * 4 and at least 128): the marching step runs work items whose entering
+ * Plateau split (FP32 contexts, for E_z ones with two columns per lane, nx a
+ * multiple of 4 and at least 128; six planes from two and a half waves of
+ * 32-row units on, about 3400^2 sites, or on any such lattice where a
+ * marching kernel but QLA_KERNEL_MARCH_PLAIN is forced and
+ * qla_set_march_tuning gives at least 16 rows): the marching step runs work items whose entering
  * sites all share one record -- a plateau of n where every site's four
  * neighbours carry its n -- four columns per lane with that record's
  * collision coefficients (no index rows, no record lookups, no potential
@@ -277,7 +280,8 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * path.  Results are bitwise those of the unsplit kernel.  The first
  * marching step after qla_set_medium or a tuning change classifies the
  * items (one small kernel and one synchronisation of the context's
- * stream), so it must not be the first call inside a stream capture.
+ * stream), so it must not be the first call inside a stream capture (six
+ * planes: such a call runs the unsplit kernel).
  * Small lattices (QLA_KERNEL_AUTO; FP32 up to about 700^2 sites, FP64 as far
  * as one tile per SM goes, double-single contexts excepted): a qla_step call
  * runs all its steps in one cooperative launch of the tile kernel, every
@@ -670,7 +674,7 @@ void qla3_destroy(qla3_ctx *ctx);
  * six-plane double-single step is two launches, one per decoupled triple). */
 long long qla_launch_count(const qla_ctx *ctx);
 
-/* The plateau plan of the FP32 E_z marching step (see qla_set_step_kernel),
+/* The plateau plan of the FP32 marching step (see qla_set_step_kernel),
  * as built for the current medium and tuning by the last marching step:
  * work items (128-column windows x row segments) per step, items run on the
  * plateau path, and distinct plateau records among them.  For a lattice whose

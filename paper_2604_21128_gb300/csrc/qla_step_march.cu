@@ -586,9 +586,10 @@ cudaError_t launch_split6(qla_ctx *c, const void *in, void *out) {
 // over the resident warp slots, each a segment with its eight halo rows, plus
 // half a segment for the tail; rows a multiple of 4, at least 16.  0 (no
 // split) below two and a half waves of 32-row units: with fewer, the units'
-// latency counts and the six-plane march, which has both triples' rotations
-// in flight per warp, is faster (us per step, march against split: 2048^2 89
-// / 102, 1536^2 69 / 64, 3000 x 1100 90 / 87 at 32 rows, 4096^2 287 / 255).
+// latency counts and the six-plane march has both triples' rotations in flight
+// per warp.  Between there and one wave it goes either way (us per step, march
+// against split at 32 rows: 1536^2 69 / 64, 3000 x 1100 90 / 87, 2048^2 89 /
+// 102); the line keeps the lattices that would lose most.  4096^2: 287 / 255.
 int split6_segment(const qla_ctx *c) {
     const long long per = 2LL * ((c->nx + PWOUT - 1) / PWOUT);
     const long long slots = 4LL * WARPS * c->num_sms;
@@ -671,16 +672,17 @@ cudaError_t launch_t(qla_ctx *c, const void *in, void *out, const void *table) {
     if constexpr (std::is_same<T, float>::value && P == 6) {
         if (c->items && c->step_kernel != QLA_KERNEL_MARCH_PLAIN && c->nx % 4 == 0 &&
             c->nx >= PW) {
-            const int sseg = c->march_seg > 0 ? std::max(16, seg) : split6_segment(c);
+            // given rows take the place of the rule's, where it splits; asked
+            // for by name, the split takes them on any lattice
+            int sseg = split6_segment(c);
+            if (c->march_seg > 0)
+                sseg = seg >= 16 && (sseg > 0 || c->step_kernel != QLA_KERNEL_AUTO) ? seg : 0;
             const auto &u = c->uplan;
             // building the plan waits for the stream: not inside a capture,
             // where the six-plane march needs no plan
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
             const bool have = u.gen == c->medium_gen && u.seg == sseg;
-            if (sseg > 0 && !have) {
-                cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-                if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone)
-                    e = ensure_plateau_plan(c, sseg, false);
+            if (sseg > 0 && !have && !capturing(c->stream)) {
+                const cudaError_t e = ensure_plateau_plan(c, sseg, false);
                 if (e != cudaSuccess) return e;
             }
             if (sseg > 0 && u.gen == c->medium_gen && u.seg == sseg && u.n_uniform > 0)

@@ -31,3 +31,26 @@ def test_six_plane_split_agrees_bitwise(nx, ny, rows, potential, split):
     assert (out["march"][2][1] > 0) == split and out["march_plain"][2] == (0, 0, 0)
     assert np.array_equal(out["march"][0], out["march_plain"][0])
     assert out["march"][1] == out["march_plain"][1]
+
+
+@pytest.mark.parametrize("kernel,rows,split", [("auto", 64, False), ("march", 64, True),
+                                               ("march", 12, False)])
+def test_rows_force_the_split_only_where_it_is_asked_for(kernel, rows, split):
+    """A lattice below the split's line (2048 x 1024): an automatic context with
+    rows set keeps the unsplit march, as does any with rows the units cannot
+    have; all give the same bits."""
+    nx, ny = 2048, 1024
+    n = np.full((ny, nx), 2.0)
+    n[:, : nx // 3] = 1.0
+    q0 = inputs.random_state(nx, ny, seed=rows)
+    out = []
+    for k, r in ((kernel, rows), ("march_plain", 0)):
+        with qla.Grid(nx, ny, 1.0, "fp32") as g:
+            g.set_step_kernel(k)
+            g.set_march_tuning(0, r)
+            g.set_medium(n)
+            g.set_state(q0)
+            g.step(3)
+            out.append((g.march_plan[1] > 0, g.get_state()))
+    assert out[0][0] == split and not out[1][0]
+    assert np.array_equal(out[0][1], out[1][1])

@@ -693,6 +693,9 @@ struct Scratch {
     }
 };
 
+// Whether the layout conversion can read a tensor's pixels (16 bytes at a time).
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // Waits for the stream; QLA_ETIMEOUT if a wait of the call's kernels ran out.
 qla_status raw_waits_ok(const int *flag_dev, cudaStream_t st) {
     int flag = 0;
@@ -708,6 +711,7 @@ extern "C" qla_status surr_conv3x3_raw(const void *in_bf16, int B, int H, int W,
                                        void *cuda_stream) {
     if (!in_bf16 || !w_bf16 || !out_f32 || B < 1 || H < 1 || W < 1 || cin % 32 || cout % 32)
         return QLA_EINVAL;
+    if (!aligned16(in_bf16)) return QLA_ECUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Scratch sx(st), sw(st), so(st), sf(st);
     bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));
@@ -745,6 +749,7 @@ extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_b
                                            float *dw_f32, void *cuda_stream) {
     if (!dz_bf16 || !in_bf16 || !part || !dw_f32 || cin % 32 || cout % 32 || splits < 1)
         return QLA_EINVAL;
+    if (!aligned16(dz_bf16) || !aligned16(in_bf16)) return QLA_ECUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Scratch sz(st), sx(st), sf(st);
     bf16 *z = sz.get<bf16>(blocked_elems(B, cout, H, W));

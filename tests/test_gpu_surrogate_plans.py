@@ -104,3 +104,29 @@ def test_gradient_with_a_wait_that_ran_out_is_refused():
     assert e.value.status == 5                     # QLA_ETIMEOUT
     got = net.loss_grad(x, t)
     assert got[0] == want[0] and np.array_equal(got[1], want[1])
+
+
+def weight_grad_raw(dz, x, B, H, W, splits=2):
+    """dz (.., cout) and x (.., cin) hold at least B H W pixels."""
+    import torch
+    cout, cin = dz.shape[-1], x.shape[-1]
+    part = torch.full((splits * cout * 9 * cin,), 7.0, device="cuda")
+    dw = torch.full((cout, 9, cin), 7.0, device="cuda")
+    st = qla.load().surr_weight_grad_raw(ctypes.c_void_p(dz.data_ptr()),
+                                         ctypes.c_void_p(x.data_ptr()), B, H, W, cout, cin, splits,
+                                         ctypes.c_void_p(part.data_ptr()),
+                                         ctypes.c_void_p(dw.data_ptr()), None)
+    torch.cuda.synchronize()
+    return st, dw
+
+
+@pytest.mark.parametrize("W", [16, 128])
+def test_tensors_off_16_byte_boundaries_are_refused(W):
+    rng = np.random.default_rng(2)
+    x, z = bf16(rng, (2 * W + 1, 32)), bf16(rng, (2 * W, 32))
+    off = x.reshape(-1)[1:1 + 2 * W * 32].reshape(1, 2, W, 32)
+    assert off.data_ptr() % 16 == 2
+    assert conv_raw(off, bf16(rng, (32, 9, 32)))[0] == 4          # QLA_ECUDA
+    off = off.reshape(-1, 32)
+    assert weight_grad_raw(z, off, 1, 2, W)[0] == 4
+    assert weight_grad_raw(off, z, 1, 2, W)[0] == 4

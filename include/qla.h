@@ -563,7 +563,7 @@ void surr_destroy(surr_net *n);
  *   dw[co][tap][ci] = sum_p dz[p][co] in[p + shift(tap)][ci]
  * with tap = 3 (dy + 1) + (dx + 1), shifts periodic in y and x; in, w, dz
  * BF16 (in and dz 16-byte aligned, else QLA_ECUDA), out and dw FP32; part
- * holds splits * cout * 9 * cin floats.  Each call
+ * holds splits * cout * 9 * cin floats; no pixels give dw = 0.  Each call
  * allocates stream-ordered scratch (cudaMallocAsync) for the network's own
  * layouts of its operands, frees it and waits for the stream (the second not
  * while the stream is being captured); QLA_ETIMEOUT if a device wait ran out. */

@@ -751,6 +751,12 @@ extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_b
         return QLA_EINVAL;
     if (!aligned16(dz_bf16) || !aligned16(in_bf16)) return QLA_ECUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (B < 1 || H < 1 || W < 1) {   // no pixels: the sums are zero
+        const size_t n = size_t(cout) * 9 * cin;
+        return cout > 0 && cin > 0 && cudaMemsetAsync(part, 0, splits * n * 4, st) == cudaSuccess &&
+                       cudaMemsetAsync(dw_f32, 0, n * 4, st) == cudaSuccess
+                   ? QLA_OK : QLA_ECUDA;
+    }
     Scratch sz(st), sx(st), sf(st);
     bf16 *z = sz.get<bf16>(blocked_elems(B, cout, H, W));
     bf16 *x = sx.get<bf16>(blocked_elems(B, cin, H, W));

@@ -120,6 +120,14 @@ def weight_grad_raw(dz, x, B, H, W, splits=2):
     return st, dw
 
 
+@pytest.mark.parametrize("B,H,W", [(0, 4, 16), (2, 0, 16), (2, 4, 0)])
+def test_weight_gradient_over_no_pixels_is_zero(B, H, W):
+    rng = np.random.default_rng(1)
+    dz, x = bf16(rng, (64, 32)), bf16(rng, (64, 64))
+    st, dw = weight_grad_raw(dz, x, B, H, W)
+    assert st == 0 and not dw.any()
+
+
 @pytest.mark.parametrize("W", [16, 128])
 def test_tensors_off_16_byte_boundaries_are_refused(W):
     rng = np.random.default_rng(2)

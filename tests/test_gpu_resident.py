@@ -39,6 +39,19 @@ def test_resident_tiles_agree_bitwise(shape, te, precision):
     assert np.array_equal(a[1], b[1]) and a[2] == b[2]
 
 
+@pytest.mark.parametrize("shape,te,kw", [((300, 301), True, {}), ((512, 500), True, {}),
+                                         ((700, 650), True, dict(potential="literal")),
+                                         ((1500, 120), True, {}), ((400, 390), False, {}),
+                                         ((330, 280), False, dict(tensor=True)),
+                                         ((333, 290), False, dict(potential="lcu"))])
+def test_several_resident_tiles_per_sm(shape, te, kw):
+    """More tiles than SMs (eight warps each), up to six per SM."""
+    a = run(shape, "auto", (4, 1, 6), "fp32", te, **kw)
+    b = run(shape, "tile", (11,), "fp32", te, **kw)
+    assert a[0] == 3 and b[0] == 11
+    assert np.array_equal(a[1], b[1]) and a[2] == b[2]
+
+
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("kw", [dict(potential="literal"), dict(potential="none"),
                                 dict(potential="lcu"), dict(te=False, potential="lcu"),

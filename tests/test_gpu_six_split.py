@@ -54,3 +54,27 @@ def test_rows_force_the_split_only_where_it_is_asked_for(kernel, rows, split):
             out.append((g.march_plan[1] > 0, g.get_state()))
     assert out[0][0] == split and not out[1][0]
     assert np.array_equal(out[0][1], out[1][1])
+
+
+def test_six_plane_split_without_a_potential():
+    test_six_plane_split_agrees_bitwise(512, 77, 20, "none", True)
+
+
+def test_automatic_six_plane_split():
+    """A lattice just above the line of split6_segment, at the height it picks."""
+    import torch
+    nx, ny = 3400, 3376
+    n = np.full((ny, nx), 2.0)
+    n[:, : nx // 3] = 1.0
+    n[-60:, -90:] = inputs.random_medium(90, 60, seed=5, lo=1.2, hi=2.8)
+    q0 = inputs.random_state(nx, ny, seed=12)
+    out = []
+    for kernel in ("auto", "march_plain"):
+        with qla.Grid(nx, ny, 1.0, "fp32") as g:
+            g.set_step_kernel(kernel)
+            g.set_medium(n)
+            g.set_state(q0)
+            g.step(3)
+            out.append((g.march_plan[1], g.pack_box(0, 0, nx, ny)))
+    assert out[0][0] > 0 and out[1][0] == 0
+    assert torch.equal(out[0][1], out[1][1])

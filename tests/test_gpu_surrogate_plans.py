@@ -28,6 +28,13 @@ def conv64(x, w):
     return out
 
 
+def accumulation_bound(steps):
+    """Relative error of a sum in `steps` K = 16 tensor-core steps: products of
+    BF16 values are exact, each step may truncate the FP32 running sum (on the
+    mean half of 2^-23 of it, the sum growing as the root of the step)."""
+    return 1e-6 + steps * 2.0 ** -24
+
+
 def conv_raw(x, w):
     import torch
     B, H, W, cin = x.shape
@@ -52,6 +59,25 @@ def test_wide_inputs_are_taken(B, H, W, cin, cout):
     # products of BF16 values are exact; the FP32 accumulation of 9 cin terms
     # rounds (~sqrt(9 cin) 6e-8 relative)
     assert float(torch.linalg.norm(out - want) / torch.linalg.norm(want)) <= 1e-5
+
+
+# (on 152 SMs) slices of 256, 128 and 64 channels, weights resident and streamed
+# in units of one, two and four patches, one tile per block and several, ragged
+# tile edges; widths of 128 take the patches in the outer loop
+@pytest.mark.parametrize("B,H,W,cin,cout", [(8, 64, 64, 256, 256), (3, 100, 90, 128, 256),
+                                            (4, 96, 96, 64, 128), (2, 130, 104, 32, 64),
+                                            (8, 128, 128, 128, 64), (2, 64, 128, 256, 128),
+                                            (1, 40, 384, 96, 160), (5, 33, 72, 160, 96),
+                                            (8, 32, 32, 128, 256), (8, 64, 64, 256, 512)])
+def test_convolution_layouts_of_large_images(B, H, W, cin, cout):
+    import torch
+    rng = np.random.default_rng(B + H + W)
+    x, w = bf16(rng, (B, H, W, cin)), bf16(rng, (cout, 9, cin), 0.1)
+    st, out = conv_raw(x, w)
+    assert st == 0
+    want = conv64(x, w)
+    assert float(torch.linalg.norm(out - want) / torch.linalg.norm(want)) <= \
+        accumulation_bound(9 * cin / 16)
 
 
 def small_net(seed=3):
@@ -118,6 +144,55 @@ def weight_grad_raw(dz, x, B, H, W, splits=2):
                                          ctypes.c_void_p(dw.data_ptr()), None)
     torch.cuda.synchronize()
     return st, dw
+
+
+# widths of part segments (48, 80, 112, 208), whole rows per stage (16, 32, with
+# heights that do and do not divide into stages), other widths; splits that end
+# within a row; 32, 16 and 8 input channels per block
+@pytest.mark.parametrize("B,H,W,cout,cin,splits", [(2, 9, 48, 32, 32, 3), (1, 17, 80, 64, 64, 5),
+                                                   (3, 11, 112, 256, 32, 2), (1, 8, 208, 32, 96, 4),
+                                                   (2, 12, 16, 64, 128, 2), (2, 6, 16, 32, 64, 3),
+                                                   (1, 10, 32, 128, 256, 3), (3, 7, 32, 96, 32, 2),
+                                                   (2, 6, 24, 64, 96, 2),
+                                                   (8, 64, 64, 256, 256, 8),
+                                                   (2, 128, 128, 64, 32, 128)])
+def test_weight_gradient_at_ragged_widths(B, H, W, cout, cin, splits):
+    import torch
+    rng = np.random.default_rng(W + cout + splits)
+    dz, x = bf16(rng, (B, H, W, cout)), bf16(rng, (B, H, W, cin))
+    st, dw = weight_grad_raw(dz, x, B, H, W, splits)
+    assert st == 0
+    want = torch.empty((cout, 9, cin), dtype=torch.float64, device="cuda")
+    z = dz.double().reshape(-1, cout).T
+    for tap in range(9):
+        shifted = torch.roll(x.double(), (1 - tap // 3, 1 - tap % 3), (1, 2))
+        want[:, tap] = z @ shifted.reshape(-1, cin)
+    assert float(torch.linalg.norm(dw - want) / torch.linalg.norm(want)) <= \
+        accumulation_bound(B * H * W / splits / 16 + 4)
+
+
+# deepest levels of one and of two pixels, sides that are no powers of two, and
+# images large enough for the wide slices; bounds: those of the small images in
+# test_gpu_surrogate.py
+@pytest.mark.parametrize("B,H,W", [(1, 16, 16), (2, 32, 16), (2, 48, 80), (1, 112, 144),
+                                   (2, 256, 128)])
+def test_network_matches_fp64_reference(B, H, W):
+    import torch
+    from oracle import surrogate as ref
+    from paper_2604_21128_gb300 import surrogate
+    net = surrogate.Surrogate(H, W, max_batch=B, seed=1)
+    rng = np.random.default_rng(H + W)
+    theta = (rng.standard_normal(net.nparams) * 0.05).astype(np.float32)
+    net.set_params(theta)
+    x, t = rng.standard_normal((B, H, W, 6)), 0.1 * rng.standard_normal((B, H, W, 3))
+    xd, td = (torch.tensor(v, dtype=torch.float32, device="cuda") for v in (x, t))
+    got = net.forward(xd).cpu().numpy()
+    want = ref.forward(theta.astype(np.float64), xd.cpu().numpy())
+    assert np.linalg.norm(got - want) <= 3e-2 * np.linalg.norm(want)
+    loss, g = net.loss_grad(xd, td)
+    rloss, rg = ref.loss_grad(theta.astype(np.float64), xd.cpu().numpy(), td.cpu().numpy())
+    assert abs(loss / rloss - 1) <= 3e-2
+    assert np.linalg.norm(g - rg) <= 5e-2 * np.linalg.norm(rg)
 
 
 @pytest.mark.parametrize("B,H,W", [(0, 4, 16), (2, 0, 16), (2, 4, 0)])

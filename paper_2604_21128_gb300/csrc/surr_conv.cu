@@ -317,7 +317,7 @@ cudaError_t launch_dw_co(const bf16 *dz, const bf16 *in, int B, const DwGeom &g,
 __global__ void __launch_bounds__(256) k_sum_splits(const __grid_constant__ SumJobs jobs) {
     __shared__ float red[256][33];
     const SumJob &j = jobs.j[blockIdx.y];
-    if (!j.tree) {
+    if (!SumJobs::tree(j)) {
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < j.n;
              i += (long long)gridDim.x * blockDim.x) {
             float s = 0.f;
@@ -656,14 +656,11 @@ cudaError_t weight_grad(const bf16 *dz, const bf16 *in, int B, int H, int W, int
 }
 
 cudaError_t sum_splits(const SumJobs &jobs, int count, cudaStream_t st) {
-    SumJobs t = jobs;
     long long most = 1;
-    for (int k = 0; k < count; ++k) {
-        t.j[k].tree = t.j[k].splits >= 64 && t.j[k].n <= 65535;
-        most = std::max(most, t.j[k].tree ? 8 * t.j[k].n : t.j[k].n);
-    }
+    for (int k = 0; k < count; ++k)
+        most = std::max(most, jobs.j[k].n * (SumJobs::tree(jobs.j[k]) ? 8 : 1));
     k_sum_splits<<<dim3(unsigned(std::min<long long>((most + 255) / 256, 1024)), unsigned(count)),
-                   256, 0, st>>>(t);
+                   256, 0, st>>>(jobs);
     return cudaGetLastError();
 }
 

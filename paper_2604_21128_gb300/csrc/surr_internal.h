@@ -60,8 +60,14 @@ int weight_grad_splits(int B, int H, int W);
 
 // Sums over splits, in a fixed order, of up to MAX_JOBS arrays in one launch.
 constexpr int MAX_JOBS = 20;
-struct SumJob { const float *part; float *dst; int splits; long long n; bool tree; };
-struct SumJobs { SumJob j[MAX_JOBS]; };
+struct SumJob { const float *part; float *dst; int splits; long long n; };
+struct SumJobs {
+    SumJob j[MAX_JOBS];
+    // many splits of few values are summed as a tree (see k_sum_splits)
+    static __host__ __device__ bool tree(const SumJob &j) {
+        return j.splits >= 64 && j.n <= 65535;
+    }
+};
 cudaError_t sum_splits(const SumJobs &jobs, int count, cudaStream_t st);
 
 // Backward through an activation: g = (source) * act'(y), dz = BF16 g, the

@@ -212,8 +212,8 @@ qla_status conv_backward(surr_net *n, int i, int B, const bf16 *dz, float *d_in,
     NCUDA(n, weight_grad(dz, conv_input(n, i), B, h, w, s.cout, s.cin, splits, n->part[i],
                          n->flag, n->stream),
           "surrogate: weight grad");
-    jobs.j[njobs++] = {n->part[i], l.gw, splits, (long long)n->nw[i], false};
-    jobs.j[njobs++] = {n->bpart[i], l.gb, bias_blocks(B, h, w), s.cout, false};
+    jobs.j[njobs++] = {n->part[i], l.gw, splits, (long long)n->nw[i]};
+    jobs.j[njobs++] = {n->bpart[i], l.gb, bias_blocks(B, h, w), s.cout};
     if (d_in) {
         ConvArgs a{};
         a.in = dz;
@@ -766,7 +766,7 @@ extern "C" qla_status surr_weight_grad_raw(const void *dz_bf16, const void *in_b
         return QLA_ECUDA;
     }
     SumJobs jobs{};
-    jobs.j[0] = {part, dw_f32, splits, (long long)cout * 9 * cin, false};
+    jobs.j[0] = {part, dw_f32, splits, (long long)cout * 9 * cin};
     if (nhwc_to_blocked(static_cast<const bf16 *>(dz_bf16), B, H, W, cout, z, st) != cudaSuccess ||
         nhwc_to_blocked(static_cast<const bf16 *>(in_bf16), B, H, W, cin, x, st) != cudaSuccess ||
         weight_grad(z, x, B, H, W, cout, cin, splits, part, flag_dev, st) != cudaSuccess ||

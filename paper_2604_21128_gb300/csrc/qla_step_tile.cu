@@ -29,11 +29,11 @@
 //
 // What bounds it: on small lattices latency (barriers, the exchange through
 // L2); with many tiles, instruction issue (FP32) or the FP64 pipe, on the
-// 1.55 x 576 sites per tile the halo costs.  Measured per step, us (start:
-// the marching kernel, or for odd sides and tensor media the tile kernel
-// this one replaces, which kept the whole region in shared memory and took
-// one barrier and one round trip through it per layer):
-//                            start   per-step tiles   resident tiles
+// 1.55 x 576 sites per tile the halo costs.  Measured per step, us (other:
+// the marching kernel, or for odd sides and tensor media a tile kernel that
+// kept the whole region in shared memory and took one barrier and one round
+// trip through it per layer):
+//                            other   per-step tiles   resident tiles
 //   256^2 FP32 E_z            16.6        6.3              3.4
 //   512^2 FP32 E_z            17.8       10.4              6.9
 //   512^2 FP32 six planes     43         14.5             10.3
@@ -470,8 +470,9 @@ cudaError_t launch_step_tile(qla_ctx *c, const void *in, void *out, bool vin) {
 
 // Which steps of an automatic context the tile kernel takes from the
 // marching one.  FP32 six planes: 1024^2 34.6 us per step against 45.2,
-// 1536^2 equal.  FP32 E_z: resident tiles only (per-step tiles 768^2 14.5 /
-// 16.6, 1024^2 22.7 / 22.7).  FP64: tiles take 0.152 to 0.170 us per 1000
+// 1536^2 equal.  FP32 E_z: resident tiles only; beyond them the march, though
+// per-step tiles win up to about 1024^2 (768^2 14.5 / 16.6, 1024^2 22.7 /
+// 22.7).  FP64: tiles take 0.152 to 0.170 us per 1000
 // sites (E_z 1024^2 to 3072^2, compared as 0.165, which leaves 1024^2, 178 /
 // 168, to the march; six planes 0.307 to 0.336, as 0.325), the march 4.2 us (8.1) per row of the items
 // that its schedulers hold one of, whatever the lattice: a march has a

@@ -272,16 +272,16 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * multiple of 4 and at least 128; six planes from two and a half waves of
  * 32-row units on, about 3400^2 sites, or on any such lattice where a
  * marching kernel but QLA_KERNEL_MARCH_PLAIN is forced and
- * qla_set_march_tuning gives at least 16 rows): the marching step runs work items whose entering
- * sites all share one record -- a plateau of n where every site's four
- * neighbours carry its n -- four columns per lane with that record's
- * collision coefficients (no index rows, no record lookups, no potential
- * step, which is the identity there); all other items take the general
- * path.  Results are bitwise those of the unsplit kernel.  The first
- * marching step after qla_set_medium or a tuning change classifies the
- * items (one small kernel and one synchronisation of the context's
- * stream), so it must not be the first call inside a stream capture (six
- * planes: such a call runs the unsplit kernel).
+ * qla_set_march_tuning gives at least 16 rows): the marching step runs work
+ * items whose entering sites all share one record -- a plateau of n where
+ * every site's four neighbours carry its n -- four columns per lane with that
+ * record's collision coefficients (no index rows, no record lookups, no
+ * potential step, which is the identity there); all other items take the
+ * general path.  Results are bitwise those of the unsplit kernel.  The first
+ * marching step after qla_set_medium or a tuning change classifies the items
+ * (one small kernel and one synchronisation of the context's stream), so it
+ * must not be the first call inside a stream capture (six planes: such a call
+ * runs the unsplit kernel).
  * Small lattices (QLA_KERNEL_AUTO; FP32 up to about 700^2 sites, FP64 as far
  * as one tile per SM goes, double-single contexts excepted): a qla_step call
  * runs all its steps in one cooperative launch of the tile kernel, every

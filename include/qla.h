@@ -290,7 +290,7 @@ qla_status qla_set_packet_window(qla_ctx *ctx, const qla_packet *p, int i0, int 
  * (qla_set_march_tuning) takes the marching kernel instead.
  * QLA_KERNEL_TILE = the tile kernel, one launch per step.
  * QLA_KERNEL_MARCH_PLAIN = the marching kernel without the split.
- * Dataflow steps (plateau split, lattices with at least about three work
+ * Dataflow steps (plateau split of E_z, lattices with about three or more work
  * items per resident warp: 16384^2 at 192-row segments, 8192^2 at 64): a
  * qla_step call runs all its steps in one persistent launch (after one
  * ordinary launch for a first step with no pending potential step).  Blocks
